@@ -81,33 +81,6 @@ int variant_index(int g, int k, int placement) {
 
 namespace {
 
-// One query by the list kind that suits its k (the thread's column holds
-// at least list_slots(k) slots). W: flag words of the kernel's k class.
-// DEFER: as knn_query_smem (false when the query was given up).
-template <int W, bool DEFER = false>
-__device__ __forceinline__ bool knn_query_smem_any(const CloudDev& C, float qx, float qy,
-                                                   float qz, int k, int m, uint64_t* col,
-                                                   int32_t* __restrict__ out_idx,
-                                                   float* __restrict__ out_d2, int32_t row) {
-  if constexpr (W == 1) {
-    if (k <= 8)
-      return knn_query_smem<SortedList<8, 1, true>, DEFER>(C, qx, qy, qz, k, m, col, 8, out_idx,
-                                                           out_d2, row);
-    else if (k <= 16)
-      return knn_query_smem<PermList16, DEFER>(C, qx, qy, qz, k, m, col, 16, out_idx, out_d2,
-                                               row);
-    else
-      return knn_query_smem<SortedList<32, 1, false>, DEFER>(C, qx, qy, qz, k, m, col, k,
-                                                             out_idx, out_d2, row);
-  } else if constexpr (W == 2) {
-    return knn_query_smem<SortedList<64, 2, false>, DEFER>(C, qx, qy, qz, k, m, col, k, out_idx,
-                                                           out_d2, row);
-  } else {
-    return knn_query_smem<SortedList<128, 4, false>, DEFER>(C, qx, qy, qz, k, m, col, k,
-                                                            out_idx, out_d2, row);
-  }
-}
-
 // This thread's column of its warp's shared-memory candidate lists.
 __device__ __forceinline__ uint64_t* smem_column(int kcap) {
   extern __shared__ uint64_t batch_lists[];
@@ -117,33 +90,45 @@ __device__ __forceinline__ uint64_t* smem_column(int kcap) {
 
 // DEFER: a query that meets a list with a box tree is handed over
 // (appended to the plan's list of its class) instead of answered.
-template <int W, bool DEFER>
+template <class L, bool DEFER>
 __device__ __forceinline__ void serve_item_smem(const ReqDev& R, const Item& w, uint64_t* col) {
   const int lane = (int)(threadIdx.x & 31u);
   const CloudDev C{R.pts, R.rows, R.succ, R.n, R.ent, DEFER ? R.hub_of : nullptr};
-  for (int i = w.begin + lane; i < w.end; i += 32) {
-    const int64_t qi = R.perm ? (int64_t)__ldg(R.perm + i) : (int64_t)i;
-    const float* qp = R.q + qi * R.q_stride;
-    const float qx = __ldg(qp), qy = __ldg(qp + 1), qz = __ldg(qp + 2);
-    const int m = R.m ? __ldg(R.m + qi) : R.m_scalar;
-    int32_t* oi = R.out_idx + qi * R.k;
-    float* od = R.out_d2 + qi * R.k;
-    if (m < 1 || m > C.n) {
-      for (int p = 0; p < R.k; ++p) {
-        oi[p] = -1;
-        od[p] = __int_as_float(0x7f800000);
+  const int k = R.k;
+  for (int i0 = w.begin; i0 < w.end; i0 += 32) {
+    const int i = i0 + lane;
+    bool live = i < w.end;
+    int64_t qi = 0;
+    float qx = 0.f, qy = 0.f, qz = 0.f;
+    int m = 0;
+    if (live) {
+      qi = R.perm ? (int64_t)__ldg(R.perm + i) : (int64_t)i;
+      const float* qp = R.q + qi * R.q_stride;
+      qx = __ldg(qp);
+      qy = __ldg(qp + 1);
+      qz = __ldg(qp + 2);
+      m = R.m ? __ldg(R.m + qi) : R.m_scalar;
+      if (m < 1 || m > C.n) {
+        live = false;
+        int32_t* oi = R.out_idx + qi * k;
+        float* od = R.out_d2 + qi * k;
+        for (int p = 0; p < k; ++p) {
+          oi[p] = -1;
+          od[p] = __int_as_float(0x7f800000);
+        }
+        atomicOr(R.err, 1);
       }
-      atomicOr(R.err, 1);
-      continue;
     }
-    const bool done =
-        knn_query_smem_any<W, DEFER>(C, qx, qy, qz, R.k, m, col, R.out_idx, R.out_d2, (int32_t)qi);
+    __syncwarp();
+    const bool gave_up = knn_query_smem<L, DEFER>(C, live, qx, qy, qz, k, m, col, R.out_idx,
+                                                  R.out_d2, (int32_t)qi);
     if constexpr (DEFER) {
-      if (!done) {
-        const int c = handover_class(R.k);
+      if (gave_up) {
+        const int c = handover_class(k);
         R.ho->list[c][atomicAdd(&R.ho->count[c], 1)] = make_int2(w.req, (int)qi);
       }
     }
+    __syncwarp();
   }
 }
 
@@ -194,7 +179,9 @@ __global__ void __launch_bounds__(kThreads, S <= 2 ? 5 : (S <= 4 ? 4 : 3)) knn_b
 
 // The one-lane variant: one query per thread, candidate lists in shared
 // memory, 256-thread blocks held to 48 registers as in the plain kernel.
-template <int THREADS, int W, bool DEFER>
+// LK: the list kind of the segment's class (8, 16 or 0), as in the plain
+// kernel.
+template <int THREADS, int W, int LK, bool DEFER>
 __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : 1) knn_batch_smem_kernel(const ReqDev* __restrict__ reqs,
                                                                  const Item* __restrict__ items,
                                                                  int nitems,
@@ -208,8 +195,12 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : 1) knn_batch_sme
     it = __shfl_sync(0xffffffffu, it, 0);
     if (it >= nitems) return;
     const Item w = items[it];
-    serve_item_smem<W, DEFER>(reqs[w.req], w, col);
-    __syncwarp();
+    if constexpr (LK == 8)
+      serve_item_smem<PermList<8>, DEFER>(reqs[w.req], w, col);
+    else if constexpr (LK == 16)
+      serve_item_smem<PermList<16>, DEFER>(reqs[w.req], w, col);
+    else
+      serve_item_smem<SortedList<32 * W, W>, DEFER>(reqs[w.req], w, col);
   }
 }
 
@@ -364,12 +355,16 @@ cudaError_t set_smem_attributes() {
   const struct {
     const void* fn;
     size_t bytes;
-  } kernels[] = {{(const void*)knn_batch_smem_kernel<256, 1, false>, list_bytes(256, 32)},
-                 {(const void*)knn_batch_smem_kernel<128, 2, false>, list_bytes(128, 64)},
-                 {(const void*)knn_batch_smem_kernel<64, 4, false>, list_bytes(64, 128)},
-                 {(const void*)knn_batch_smem_kernel<256, 1, true>, list_bytes(256, 32)},
-                 {(const void*)knn_batch_smem_kernel<128, 2, true>, list_bytes(128, 64)},
-                 {(const void*)knn_batch_smem_kernel<64, 4, true>, list_bytes(64, 128)}};
+  } kernels[] = {{(const void*)knn_batch_smem_kernel<256, 1, 8, false>, list_bytes(256, 8)},
+                 {(const void*)knn_batch_smem_kernel<256, 1, 16, false>, list_bytes(256, 16)},
+                 {(const void*)knn_batch_smem_kernel<256, 1, 0, false>, list_bytes(256, 32)},
+                 {(const void*)knn_batch_smem_kernel<128, 2, 0, false>, list_bytes(128, 64)},
+                 {(const void*)knn_batch_smem_kernel<64, 4, 0, false>, list_bytes(64, 128)},
+                 {(const void*)knn_batch_smem_kernel<256, 1, 8, true>, list_bytes(256, 8)},
+                 {(const void*)knn_batch_smem_kernel<256, 1, 16, true>, list_bytes(256, 16)},
+                 {(const void*)knn_batch_smem_kernel<256, 1, 0, true>, list_bytes(256, 32)},
+                 {(const void*)knn_batch_smem_kernel<128, 2, 0, true>, list_bytes(128, 64)},
+                 {(const void*)knn_batch_smem_kernel<64, 4, 0, true>, list_bytes(64, 128)}};
   cudaError_t e = cudaSuccess;
   for (const auto& kn : kernels)
     if (e == cudaSuccess)
@@ -386,8 +381,17 @@ cudaError_t ensure_smem_attributes() {
   });
 }
 
-// The kernel of a variant (the one-lane kernel by its block size).
-const void* variant_kernel(int variant, int threads) {
+// The one-lane kernel of a list capacity (list_slots of the segment's k).
+template <bool DEFER>
+const void* smem_kernel(int kcap) {
+  if (kcap <= 8) return (const void*)knn_batch_smem_kernel<256, 1, 8, DEFER>;
+  if (kcap <= 16) return (const void*)knn_batch_smem_kernel<256, 1, 16, DEFER>;
+  if (kcap <= 32) return (const void*)knn_batch_smem_kernel<256, 1, 0, DEFER>;
+  return (const void*)knn_batch_smem_kernel<128, 2, 0, DEFER>;
+}
+
+// The kernel of a variant (the one-lane kernel by its list capacity).
+const void* variant_kernel(int variant, int kcap) {
   switch (variant) {
     case 0: return (const void*)knn_batch_group_kernel<4, 1>;
     case 1: return (const void*)knn_batch_group_kernel<4, 2>;
@@ -409,14 +413,10 @@ const void* variant_kernel(int variant, int threads) {
     case kTreeVariant32: return (const void*)knn_batch_warp_kernel<32, true>;
     case kTreeVariant32 + 1: return (const void*)knn_batch_warp_kernel<64, true>;
     case kTreeVariant32 + 2: return (const void*)knn_batch_warp_kernel<128, true>;
-    case kSmemVariant:
-      return threads == 256 ? (const void*)knn_batch_smem_kernel<256, 1, false>
-                            : (const void*)knn_batch_smem_kernel<128, 2, false>;
-    case kSmemVariant128: return (const void*)knn_batch_smem_kernel<64, 4, false>;
-    case kHandoverVariant:
-      return threads == 256 ? (const void*)knn_batch_smem_kernel<256, 1, true>
-                            : (const void*)knn_batch_smem_kernel<128, 2, true>;
-    case kHandoverVariant128: return (const void*)knn_batch_smem_kernel<64, 4, true>;
+    case kSmemVariant: return smem_kernel<false>(kcap);
+    case kSmemVariant128: return (const void*)knn_batch_smem_kernel<64, 4, 0, false>;
+    case kHandoverVariant: return smem_kernel<true>(kcap);
+    case kHandoverVariant128: return (const void*)knn_batch_smem_kernel<64, 4, 0, true>;
     default: return nullptr;
   }
 }
@@ -432,7 +432,7 @@ BatchLaunch batch_config(int nitems, int blocks_per_sm, int kcap, int variant) {
   b.threads = is_smem128_variant(variant) ? 64 : smem ? (kcap <= 32 ? 256 : 128) : kThreads;
   b.smem = smem ? list_bytes(b.threads, kcap) : 0;
   int occ = 1;
-  const void* fn = variant_kernel(variant, b.threads);
+  const void* fn = variant_kernel(variant, b.kcap);
   if (!fn || cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, b.threads, b.smem) !=
                  cudaSuccess || occ < 1) {
     cudaGetLastError();
@@ -450,7 +450,7 @@ cudaError_t launch_batch_kernel(const ReqDev* d_reqs, const Item* d_items, int n
   if (nitems <= 0) return cudaSuccess;
   const cudaError_t ae = ensure_smem_attributes();
   if (ae != cudaSuccess) return ae;
-  const void* fn = variant_kernel(b.variant, b.threads);
+  const void* fn = variant_kernel(b.variant, b.kcap);
   if (!fn) return cudaErrorInvalidValue;
   int kcap = b.kcap;
   void* args[] = {(void*)&d_reqs, (void*)&d_items, (void*)&nitems, (void*)&d_next, (void*)&kcap};

@@ -329,7 +329,7 @@ mknn_status mknn_cloud_upload(mknn_cloud* c, mknn_stream_t stream) {
   if ((e = cudaMalloc(&c->d_pts, b_pts)) != cudaSuccess ||
       (e = cudaMalloc((void**)&c->d_rows, b_rows)) != cudaSuccess ||
       (e = cudaMalloc((void**)&c->d_succ, b_succ)) != cudaSuccess ||
-      (e = cudaMalloc(&c->d_ent, b_ent)) != cudaSuccess ||
+      (e = cudaMalloc(&c->d_ent, ent_bytes(ecap))) != cudaSuccess ||
       (e = cudaMalloc((void**)&c->d_err, 256)) != cudaSuccess) {
     cudaGetLastError();
     free_device(c);

@@ -99,6 +99,9 @@ namespace mknn {
 // Empty slots left after every row of a dynamic cloud when its table is laid
 // out (upload, compaction), so that most rows take a few appends in place.
 constexpr int64_t kRowSlack = 2;
+// Bytes of an inlined entry table of `cap` slots: the kernels read entries in
+// aligned pairs, so the last pair may reach one slot past the last entry.
+inline size_t ent_bytes(int64_t cap) { return ((size_t)cap + 1) * 16; }
 // Writes the cloud's CSR into device arrays, `slack` empty slots after each
 // row (row i starts at rowp[i] + slack * i), and fills ent from it.
 cudaError_t upload_entries(const mknn_cloud* c, int32_t* d_succ, void* d_ent, int64_t slack,

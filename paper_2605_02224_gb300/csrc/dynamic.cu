@@ -126,7 +126,7 @@ mknn_status update_device(mknn_cloud* c, int64_t n_old,
                                           (int64_t)0x7FFFFFFE);
     const size_t keep = (size_t)c->ent_cap;
     if ((e = grow((void**)&c->d_succ, keep * 4, (size_t)cap * 4, s)) != cudaSuccess ||
-        (e = grow(&c->d_ent, keep * 16, (size_t)cap * 16, s)) != cudaSuccess)
+        (e = grow(&c->d_ent, keep * 16, ent_bytes(cap), s)) != cudaSuccess)
       return afail(MKNN_ENOMEM, std::string("growing the entry arena: ") + cudaGetErrorString(e));
     c->dev_bytes += (size_t)(cap - c->ent_cap) * 20;
     c->ent_cap = cap;
@@ -192,7 +192,7 @@ mknn_status compact_device(mknn_cloud* c, cudaStream_t s) {
   void* ent = nullptr;
   cudaError_t e;
   if ((e = cudaMalloc((void**)&succ, (size_t)cap * 4)) != cudaSuccess ||
-      (e = cudaMalloc(&ent, (size_t)cap * 16)) != cudaSuccess) {
+      (e = cudaMalloc(&ent, ent_bytes(cap))) != cudaSuccess) {
     cudaGetLastError();
     cudaFree(succ);
     return afail(MKNN_ENOMEM, std::string("compacting the entry arena: ") + cudaGetErrorString(e));

@@ -530,30 +530,25 @@ __device__ __forceinline__ void knn_query_thread(const CloudDev& C, float qx, fl
 // One query per thread with the candidate list N in shared memory: entry i
 // of the lane's list at col[i * 32] (a warp's lists interleaved, so any mix
 // of positions across the lanes is bank-conflict free). An entry is one
-// 64-bit key, the float bits of the squared distance above the rank:
-// distances are never negative, so the integer order of the keys is the
-// (distance, rank) order and a comparison, a load or a move is one
-// instruction. Slots not yet filled hold a pad key above every real one,
-// so the search for an insertion position is a fixed sequence of halving
-// steps with no bound to track. The search also finds an equal key, so the
-// membership test of Alg. 2 costs nothing extra. The nearest not-yet-
+// 64-bit key, the float bits of the squared distance above the rank plus
+// one: distances are never negative, so the integer order of the keys is
+// the (distance, rank) order and a comparison, a load or a move is one or
+// two instructions. Slots not yet filled hold a pad key above every real
+// one, so the search for an insertion position is a fixed sequence of
+// halving steps with no bound to track. The search also finds an equal key,
+// so the membership test of Alg. 2 costs nothing extra. The nearest not-yet-
 // expanded entry among the first k-1 is one bit scan of the expanded mask;
 // the output comes out in order. The list takes no registers, which leaves
 // room for more resident warps.
 //
 // The lanes of a warp run in step, so the warp pays for the insertion code
-// whenever any of its lanes inserts (about one entry in five offers a
-// candidate below the k-th key, half of them already in N): insertion is
-// kept to a short sequence with no data-dependent loop where that pays.
-//  * SortedList: keys kept in position order; an insertion shifts the tail
-//    by one slot (a loop as long as the longest shift among the lanes
-//    inserting). Used where lists are short (k <= 8) or long (k > 16).
-//  * PermList16 (9 <= k <= 16): keys stay in the slot they were written to;
-//    a 64-bit register holds the slot of each position, four bits each. An
-//    insertion writes the new key into the slot of position k-1 (the
-//    dropped key, or a pad) and moves that slot's four bits to the
-//    insertion position: no key moves, a fixed instruction sequence
-//    (measured 1.10x the sorted list at k = 16, 0.97x at k = 8).
+// whenever any of its lanes inserts: insertion is kept to a short sequence
+// with no data-dependent loop where that pays.
+//  * PermList<8> (k <= 8), PermList<16> (k <= 16): keys stay where they were
+//    written, a register holds their order.
+//  * SortedList (k > 16): keys kept in position order; an insertion shifts
+//    the tail by one slot (a loop as long as the longest shift among the
+//    lanes inserting).
 __device__ __forceinline__ uint64_t pack_key(float d, uint32_t r) {
   return ((uint64_t)__float_as_uint(d) << 32) | r;
 }
@@ -629,10 +624,13 @@ __device__ __forceinline__ void flags_set(Flags<W>& F, int pos) {
   }
 }
 
+// A one-lane list's key: the rank is stored plus one, so that 0 is below
+// every real key.
+__device__ __forceinline__ uint64_t lane_key(float d, int s) { return pack_key(d, (uint32_t)s + 1u); }
+
 // Keys in position order. KS: the search size (a power of two >= the
-// list's capacity cap); positions in [cap, KS) read as pads without a load
-// unless EXACT (cap == KS).
-template <int KS, int W, bool EXACT>
+// list's capacity cap); positions in [cap, KS) read as pads without a load.
+template <int KS, int W>
 struct SortedList {
   uint64_t* col;
   int cap;
@@ -640,9 +638,9 @@ struct SortedList {
   Flags<W> done;   // bit i: entry at position i expanded
   uint64_t worst;  // key of position k-1 (a pad while cnt < k)
 
-  __device__ __forceinline__ void init(uint64_t* c, int capacity) {
+  __device__ __forceinline__ void init(uint64_t* c, int k) {
     col = c;
-    cap = EXACT ? KS : capacity;
+    cap = k;
     cnt = 0;
     done = Flags<W>{};
     worst = kPadKey;
@@ -650,7 +648,7 @@ struct SortedList {
   }
   __device__ __forceinline__ uint64_t key_at(int pos) const { return col[pos * 32]; }
   __device__ __forceinline__ uint64_t probe(int pos) const {
-    return (EXACT || pos < cap) ? col[pos * 32] : kPadKey;
+    return pos < cap ? col[pos * 32] : kPadKey;
   }
   // Inserts key c unless present; requires c < worst (then the position
   // found is below k <= cap).
@@ -666,48 +664,91 @@ struct SortedList {
     if (cnt < k) cnt++;
     if (cnt == k) worst = col[(k - 1) * 32];
   }
+  // Marks the nearest entry among the first k-1 not yet expanded and
+  // returns its rank, or -1 when there is none.
+  __device__ __forceinline__ int next(int k) {
+    const int pos = flags_first_clear(done, min(cnt, k - 1));
+    if (pos < 0) return -1;
+    flags_set(done, pos);
+    return (int)((uint32_t)col[pos * 32] - 1u);
+  }
 };
 
-// 9 <= k <= 16: sixteen slots, the order held in a register (see above).
-struct PermList16 {
-  uint64_t* col;
-  uint64_t perm;   // bits 4j..4j+3: the slot of position j
-  int cnt;
-  Flags<1> done;   // by position
-  uint64_t worst;  // key of position k-1 (a pad while cnt < k)
+template <int S>
+struct PermWord;
+template <>
+struct PermWord<8> {
+  using T = uint32_t;
+  static constexpr T identity = 0x76543210u;
+};
+template <>
+struct PermWord<16> {
+  using T = uint64_t;
+  static constexpr T identity = 0xFEDCBA9876543210ull;
+};
 
-  __device__ __forceinline__ void init(uint64_t* c, int) {
+// S = 8 (k <= 8) or 16 (k <= 16) slots: keys stay in the slot they were
+// written to; a register holds the slot of each position, four bits each.
+// The list's k positions are the last k of S: the first S - k hold key 0
+// (below every real key, marked expanded), so the position that drops out
+// is always S - 1 and no step depends on k. An insertion writes the new key
+// into the slot of position S - 1 and moves that slot's four bits to the
+// insertion position: no key moves, a fixed instruction sequence.
+template <int S>
+struct PermList {
+  using T = typename PermWord<S>::T;
+  uint64_t* col;
+  T perm;          // bits 4j..4j+3: the slot of position j
+  uint32_t done;   // by position
+  uint64_t worst;  // key of position S-1 (a pad while fewer than k entries)
+
+  __device__ __forceinline__ void init(uint64_t* c, int k) {
     col = c;
-    perm = 0xFEDCBA9876543210ull;
-    cnt = 0;
-    done = Flags<1>{};
+    perm = PermWord<S>::identity;
+    done = (1u << (S - k)) - 1u;
     worst = kPadKey;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) col[i * 32] = kPadKey;
+    for (int i = 0; i < S; ++i) col[i * 32] = i < S - k ? 0ull : kPadKey;
   }
-  __device__ __forceinline__ int slot(int pos) const { return (int)((perm >> (4 * pos)) & 15ull); }
-  __device__ __forceinline__ uint64_t key_at(int pos) const { return col[slot(pos) * 32]; }
-  // Inserts key c unless present; requires c < worst and 9 <= k <= 16.
-  __device__ __forceinline__ void insert(uint64_t c, int k) {
-    int pos = 0;
+  // the key whose slot is the four bits of perm at bit sh
+  __device__ __forceinline__ uint64_t at(int sh) const {
+    return col[((uint32_t)(perm >> sh) & 15u) * 32];
+  }
+  __device__ __forceinline__ uint64_t key_at(int pos, int k) const { return at(4 * (S - k + pos)); }
+  // Inserts key c unless present; requires c < worst.
+  __device__ __forceinline__ void insert(uint64_t c, int) {
+    int sh = 0;  // four times the number of keys below c
 #pragma unroll
-    for (int step = 8; step >= 1; step >>= 1)
-      if (col[slot(pos + step - 1) * 32] < c) pos += step;
-    // pos <= k - 1 because c < worst; slot() is below 16 whatever pos is, so
-    // no access leaves the thread's sixteen slots
-    if (col[slot(pos) * 32] == c) return;
-    const int w = slot(k - 1);  // the dropped key's slot (or a pad's)
+    for (int step = S / 2; step >= 1; step >>= 1)
+      if (at(sh + 4 * (step - 1)) < c) sh += 4 * step;
+    if (at(sh) == c) return;
+    const uint32_t w = (uint32_t)(perm >> (4 * S - 4));  // the dropped key's slot (or a pad's)
     col[w * 32] = c;
-    // positions pos..k-2 move up by one, w goes to pos, k..15 stay
-    const uint64_t below = pos ? (~0ull >> (64 - 4 * pos)) : 0ull;
-    const uint64_t live = (k == 16) ? ~0ull : (~0ull >> (64 - 4 * k));
-    const uint64_t mid = perm & live & ~below & ~(15ull << (4 * (k - 1)));
-    perm = (perm & below) | ((uint64_t)w << (4 * pos)) | (mid << 4) | (perm & ~live);
-    flags_insert(done, pos);
-    if (cnt < k) cnt++;
-    if (cnt == k) worst = (pos == k - 1) ? c : col[slot(k - 1) * 32];
+    // positions from sh / 4 on move up by one, w goes to sh / 4
+    const T low = perm & ((T(1) << sh) - 1);
+    perm = low | ((perm ^ low) << 4) | (T(w) << sh);
+    const uint32_t fl = done & ((1u << (sh >> 2)) - 1u);
+    done = fl | ((done ^ fl) << 1);
+    worst = at(4 * S - 4);
+  }
+  __device__ __forceinline__ int next(int) {
+    const uint32_t c = ~done & ((1u << (S - 1)) - 1u);
+    if (c == 0u) return -1;
+    const int pos = __ffs((int)c) - 1;
+    const uint64_t key = at(4 * pos);
+    if (key == kPadKey) return -1;  // pads only from here on
+    done |= 1u << pos;
+    return (int)((uint32_t)key - 1u);
   }
 };
+template <int KS, int W>
+__device__ __forceinline__ uint64_t list_key(const SortedList<KS, W>& N, int p, int) {
+  return N.key_at(p);
+}
+template <int S>
+__device__ __forceinline__ uint64_t list_key(const PermList<S>& N, int p, int k) {
+  return N.key_at(p, k);
+}
 
 // Descent decision: is the candidate at squared distance d (site ps)
 // strictly closer than the current site (dcur, pc)? float32 outside the
@@ -723,110 +764,182 @@ __device__ __forceinline__ bool strictly_closer(float qx, float qy, float qz, fl
   return sqd64(qx, qy, qz, ps.x, ps.y, ps.z) < sqd64(qx, qy, qz, pc.x, pc.y, pc.z);
 }
 
-// strictly_closer with the current site given by its rank: its coordinates
-// are loaded only when the float32 decision is inside the guard band.
+// strictly_closer with both sites given by their ranks: the coordinates are
+// loaded only when the float32 decision is inside the guard band.
 __device__ __forceinline__ bool strictly_closer_at(const CloudDev& C, float qx, float qy, float qz,
-                                                   float d, float4 ps, float dcur, int cur) {
+                                                   float d, int s, float dcur, int cur) {
   if (dcur >= kTiny) {
     if (d < dcur * (1.f - kGuard)) return true;
     if (d > dcur * (1.f + kGuard)) return false;
   } else if (d > 2.f * kTiny) {
     return false;
   }
-  const float4 pc = __ldg(C.pts + cur);
+  const float4 ps = __ldg(C.pts + s), pc = __ldg(C.pts + cur);
   return sqd64(qx, qy, qz, ps.x, ps.y, ps.z) < sqd64(qx, qy, qz, pc.x, pc.y, pc.z);
 }
 
-// Algorithms 1 and 2 for one query as one flat loop: each iteration either
-// consumes one successor entry (a descent step while descending, an offer
-// to N while expanding) or moves to the next row (a descent move, the end
-// of the descent, or the nearest list not yet expanded). The threads of a
-// warp then advance entry by entry together whatever their row lengths,
-// instead of waiting at the end of every row for the longest one (measured
-// 1.3x-2x faster than the row-by-row loop nest). Entries come from the
-// inlined table (site and rank in one 16-byte load), the next one loaded
-// one iteration ahead. L is a SortedList or PermList16 over the thread's
-// column col, with `cap` slots.
+// Two consecutive entries of the inlined table (the first at an even index)
+// in one 32-byte load.
+__device__ __forceinline__ void load_pair(const float4* p, float4& a, float4& b) {
+  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+      : "l"(p));
+}
+
+// Algorithms 1 and 2 for the 32 queries of a warp, one per lane, in two
+// alternating phases.
 //
-// DEFER (a cloud with box trees over its long lists, hub_of not NULL): the
-// query gives up, returning false with nothing written, when it would read
-// a list with a tree through - the expansion of such a list, or a descent
-// that finds no strictly closer entry among its first kHubScanFirst - so
-// that the one-warp kernel, which walks the tree instead, answers it; the
-// queries that never meet such a list (most of them) stay on one lane.
+// Scan: every lane with nothing to do reads its row two entries at a time
+// and stops at the first pair with something to do: an entry that passes
+// the float32 bound thr (descent: it may be strictly closer; expansion: it
+// may be below the k-th key), or the row's end. Event: all such lanes act
+// together - the hit is decided exactly and inserted, the descent moves, the
+// next list not yet expanded is opened.
+//
+// Why two phases: the kernel is bound by instruction issue and divergence.
+// With one loop over entries (test, insertion and row switch in every
+// iteration) a warp of the 4M-query torus batch ran the insertion code in
+// 72% of its 586 iterations with about 7 lanes in it, and 10.3 of 32 lanes
+// were active per instruction. Waiting until two thirds of the lanes have
+// something to do runs the event code about 190 times with 16 or more
+// lanes. A third to three quarters of the lanes measure within 5% of each
+// other; a bounded number of scan steps keeps the waiting lanes from
+// standing by while one lane reads a list of thousands (plan of 12 clouds:
+// 4.50 ms with 8 steps, 5.97 ms unbounded; 3 / 5 / 8 / 16 steps on the
+// torus batch: 6.19 / 6.07 / 6.04 / 6.05 ms).
+//
+// Why pairs: entries come from the inlined table (site and rank in 16
+// bytes), two in one 32-byte load at an even index, the next pair in flight
+// while the current one is tested: half the load instructions and half the
+// L1 lines touched (8,700 to 4,600 per warp; L1 takes about one line per
+// cycle). A pair may begin before the row (skip) or reach past its end.
+//
+// 4M queries, 1M-site torus, k = 16: 9.12 ms with the one-loop form, 6.04 ms
+// now; 1M queries, 300k-site bumpy sphere, k = 4: 0.98 to 0.58 ms.
+//
+// DEFER (a cloud with box trees over its long lists, hub_of not NULL): a
+// query gives up, with nothing written (the function returns true), when it
+// would read a list with a tree through - the expansion of such a list, or
+// a descent that finds no strictly closer entry among its first
+// kHubScanFirst - so that the one-warp kernel, which walks the tree
+// instead, answers it; the queries that never meet such a list (most of
+// them) stay on one lane.
+//
+// Called by the whole warp; lanes without a query pass live = false.
 template <class L, bool DEFER = false>
-__device__ __forceinline__ bool knn_query_smem(const CloudDev& C, float qx, float qy, float qz,
-                                               int k, int m, uint64_t* col, int cap,
+__device__ __forceinline__ bool knn_query_smem(const CloudDev& C, bool live, float qx, float qy,
+                                               float qz, int k, int m, uint64_t* col,
                                                int32_t* __restrict__ out_idx,
                                                float* __restrict__ out_d2, int32_t row) {
-  // an entry past the end of a row: rank bits 0x7fffffff, never < m
-  const float4 kNone = make_float4(0.f, 0.f, 0.f, __int_as_float(0x7fffffff));
+  // a lane's event: hits of its last pair still to be decided, the end of
+  // its row (handled once no hit is left); kIdle alone: no query (any more)
+  constexpr uint32_t kHit0 = 1u, kHit1 = 2u, kRowEnd = 4u, kIdle = 8u;
+  constexpr int kScanSteps = 8;
   L N;
-  N.init(col, cap);
+  N.init(col, k);
   float dcur = sqd32(qx, qy, qz, __ldg(C.pts));
-  N.insert(pack_key(dcur, 0u), k);
-  // rank of the descent's current site, -1 once the descent is over (its
-  // coordinates are reloaded only for a float64 recheck, which is rare)
-  int cur = 0;
-  int2 rr = __ldg(C.rows);
-  // DEFER: the current list has a tree and its scan stops after
-  // kHubScanFirst entries
-  bool cut = false;
-  if constexpr (DEFER) {
-    if (__ldg(C.hub_of) >= 0) {
-      cut = rr.y > rr.x + kHubScanFirst;
-      rr.y = min(rr.y, rr.x + kHubScanFirst);
-    }
-  }
-  int e = rr.x, end = rr.y;
-  float4 next = e < end ? __ldg(C.ent + e) : kNone;
-  for (;;) {
-    const int s = __float_as_int(next.w);
-    if (s < m) {  // the row's next entry exists and is in the prefix
-      const float4 ps = next;
-      ++e;
-      next = e < end ? __ldg(C.ent + e) : kNone;
-      const float d = sqd32(qx, qy, qz, ps);
-      const uint64_t key = pack_key(d, (uint32_t)s);
-      if (cur >= 0) {
-        if (strictly_closer_at(C, qx, qy, qz, d, ps, dcur, cur)) {
-          dcur = d;
-          cur = s;
-          if (key < N.worst) N.insert(key, k);
-          rr = __ldg(C.rows + s);
-          if constexpr (DEFER) {
-            cut = false;
-            if (__ldg(C.hub_of + s) >= 0) {
-              cut = rr.y > rr.x + kHubScanFirst;
-              rr.y = min(rr.y, rr.x + kHubScanFirst);
-            }
-          }
-          e = rr.x;
-          end = rr.y;
-          next = e < end ? __ldg(C.ent + e) : kNone;
-        }
-      } else if (key < N.worst) {
-        N.insert(key, k);
+  N.insert(lane_key(dcur, 0), k);
+  float thr = dcur >= kTiny ? dcur * (1.f + kGuard) : 2.f * kTiny;
+  int cur = 0;         // the descent's current site, -1 once it is over
+  // (its coordinates are loaded only for a float64 recheck, which is rare)
+  bool gave_up = false;
+  bool cut = false;    // DEFER: the current list has a tree and its scan stops early
+  uint32_t ev = kIdle;
+  int e = 0, end = 0, skip = 0;
+  float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
+  float d0 = 0.f, d1 = 0.f;
+  int s0 = 0, s1 = 0;
+  int open = live ? 0 : -1;  // the site whose list is read next
+  uint32_t act = __ballot_sync(0xffffffffu, live);
+  const auto open_row = [&]() {
+    int2 rr = __ldg(C.rows + open);
+    if constexpr (DEFER) {
+      cut = false;
+      if (__ldg(C.hub_of + open) >= 0) {
+        cut = rr.y > rr.x + kHubScanFirst;
+        rr.y = min(rr.y, rr.x + kHubScanFirst);
       }
-      continue;
     }
-    // the current row is done: no closer site in it (descent), or fully offered
-    if constexpr (DEFER) {
-      if (cut && e >= end) return false;  // the descent's scan was cut short
-    }
-    cur = -1;
-    const int pos = flags_first_clear(N.done, min(N.cnt, k - 1));
-    if (pos < 0) break;
-    flags_set(N.done, pos);
-    const int site = (int)(uint32_t)N.key_at(pos);
-    if constexpr (DEFER) {
-      if (__ldg(C.hub_of + site) >= 0) return false;  // an expansion of a list with a tree
-    }
-    rr = __ldg(C.rows + site);
-    e = rr.x;
     end = rr.y;
-    next = e < end ? __ldg(C.ent + e) : kNone;
+    skip = rr.x & 1;
+    e = rr.x - skip;
+    open = -1;
+    ev = kRowEnd;
+    if (rr.x < end) {
+      load_pair(C.ent + e, a, b);
+      ev = 0u;
+    }
+  };
+  if (open >= 0) open_row();
+  while (act) {
+    const int na = __popc(act);
+    for (int step = 0; step < kScanSteps; ++step) {
+      const uint32_t waiting = __ballot_sync(0xffffffffu, ev != 0u) & act;
+      if (3 * __popc(waiting) >= 2 * na) break;
+      if (ev == 0u) {
+        d0 = sqd32(qx, qy, qz, a);
+        d1 = sqd32(qx, qy, qz, b);
+        s0 = __float_as_int(a.w);
+        s1 = __float_as_int(b.w);
+        const bool more = e + 2 < end && s1 < m;
+        if (!skip && s0 < m && !(d0 > thr)) ev = kHit0;
+        if (e + 1 < end && s1 < m && !(d1 > thr)) ev |= kHit1;
+        skip = 0;
+        if (more) {
+          e += 2;
+          load_pair(C.ent + e, a, b);
+        } else {
+          ev |= kRowEnd;
+        }
+      }
+    }
+    if (ev != 0u && ev != kIdle) {
+      if (ev & (kHit0 | kHit1)) {
+        const bool first = ev & kHit0;
+        const float d = first ? d0 : d1;
+        const int s = first ? s0 : s1;
+        ev &= first ? ~kHit0 : ~kHit1;
+        const uint64_t key = lane_key(d, s);
+        bool offer = true;
+        if (cur >= 0) {
+          offer = strictly_closer_at(C, qx, qy, qz, d, s, dcur, cur);
+          if (offer) {
+            dcur = d;
+            cur = s;
+            open = s;
+            ev = 0u;
+            thr = dcur >= kTiny ? dcur * (1.f + kGuard) : 2.f * kTiny;
+          }
+        }
+        if (offer && key < N.worst) {
+          N.insert(key, k);
+          if (cur < 0) thr = __uint_as_float((uint32_t)(N.worst >> 32));
+        }
+      }
+      if (ev == kRowEnd) {
+        bool stop = false;
+        if constexpr (DEFER) {
+          if (cut) stop = !((e + 1 < end ? s1 : s0) >= m);  // the descent's scan was cut short
+        }
+        if (!stop) {
+          cur = -1;
+          thr = __uint_as_float((uint32_t)(N.worst >> 32));
+          open = N.next(k);
+          if constexpr (DEFER) {
+            if (open >= 0 && __ldg(C.hub_of + open) >= 0) stop = true;
+          }
+        }
+        if (DEFER && stop) {
+          gave_up = true;
+          open = -1;
+        }
+        if (open < 0) ev = kIdle;
+      }
+      if (open >= 0) open_row();
+    }
+    act = __ballot_sync(0xffffffffu, ev != kIdle);
   }
+  if (!live || gave_up) return gave_up;
   // the output row is addressed only now, from its 32-bit index (fewer
   // registers held through the loop); streaming stores, so that the rows
   // written do not push successor entries out of L2; four values per
@@ -842,9 +955,9 @@ __device__ __forceinline__ bool knn_query_smem(const CloudDev& C, float qx, floa
       float dv[4];
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
-        const bool real = p + t < N.cnt;
-        const uint64_t key = real ? N.key_at(p + t) : 0ull;
-        iv[t] = real ? (int32_t)(uint32_t)key : -1;
+        const uint64_t key = list_key(N, p + t, k);
+        const bool real = key != kPadKey;
+        iv[t] = real ? (int32_t)((uint32_t)key - 1u) : -1;
         dv[t] = real ? __uint_as_float((uint32_t)(key >> 32)) : __int_as_float(0x7f800000);
       }
       __stcs(reinterpret_cast<int4*>(oi + p), make_int4(iv[0], iv[1], iv[2], iv[3]));
@@ -852,13 +965,13 @@ __device__ __forceinline__ bool knn_query_smem(const CloudDev& C, float qx, floa
     }
   } else {
     for (int p = 0; p < k; ++p) {
-      const bool real = p < N.cnt;
-      const uint64_t key = real ? N.key_at(p) : 0ull;
-      __stcs(oi + p, real ? (int32_t)(uint32_t)key : -1);
+      const uint64_t key = list_key(N, p, k);
+      const bool real = key != kPadKey;
+      __stcs(oi + p, real ? (int32_t)((uint32_t)key - 1u) : -1);
       __stcs(od + p, real ? __uint_as_float((uint32_t)(key >> 32)) : __int_as_float(0x7f800000));
     }
   }
-  return true;
+  return false;
 }
 
 // Slots of a thread's list column for k: 8 for k <= 8, 16 for k <= 16 (the
@@ -1130,7 +1243,7 @@ __device__ __forceinline__ int hub_first_closer(const CloudDev& C, int hub, floa
         const float4 ps = __ldg(C.hub_ent + D.x + 32 * chunk + lane);
         const int s = __float_as_int(ps.w);  // pads: 0x7fffffff, never below m
         const float d = sqd32(qx, qy, qz, ps);
-        const bool cl = s < m && s < best && strictly_closer_at(C, qx, qy, qz, d, ps, dcur, cur);
+        const bool cl = s < m && s < best && strictly_closer_at(C, qx, qy, qz, d, s, dcur, cur);
         const int low = __reduce_min_sync(0xffffffffu, cl ? s : 0x7fffffff);
         if (low < best) {
           const int w = __ffs((int)__ballot_sync(0xffffffffu, cl && s == low)) - 1;
@@ -1235,7 +1348,7 @@ __device__ __forceinline__ void knn_query_warp(const CloudDev& C, float qx, floa
       const uint64_t key = pack_key(d, (uint32_t)s);
       const bool row_done = __any_sync(0xffffffffu, valid && !inr) || base + 32 >= end;
       if (cur >= 0) {
-        const bool cl = inr && strictly_closer_at(C, qx, qy, qz, d, ps, dcur, cur);
+        const bool cl = inr && strictly_closer_at(C, qx, qy, qz, d, s, dcur, cur);
         const uint32_t b = __ballot_sync(0xffffffffu, cl);
         if (b) {
           const int w = __ffs((int)b) - 1;

@@ -113,8 +113,8 @@ cudaError_t run_thread(const CloudDevHost& c, const PlainLaunch& L, cudaStream_t
 // held to 48 registers (five blocks per SM, no spills): left alone the
 // compiler picks either 40 registers with spills or 64, both measured
 // 5%-20% slower, and 4 or 6 blocks per SM were slower too.
-// LK: the list kind (8: SortedList of 8 slots, k <= 8; 16: PermList16,
-// 9 <= k <= 16; 0: SortedList of k slots searched over 32 W). DEFER (a
+// LK: the list kind (8: PermList<8>, k <= 8; 16: PermList<16>, 9 <= k <= 16;
+// 0: SortedList of k slots searched over 32 W). DEFER (a
 // cloud with box trees): a query that gives up (knn_query_smem) is appended
 // to defer[0 .. *ndefer) for the one-warp kernel.
 template <int THREADS, int W, int LK, bool DEFER>
@@ -129,39 +129,46 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : 1) knn_plain_sme
   // 32-bit query indices keep registers free for residency; unsigned, so
   // that i + stride cannot overflow (nq < 2^31 - 1, stride < 2^31).
   // The lanes of a warp take adjacent queries of the locality order and
-  // start their next ones together: a lane done early waits at the inner
-  // loop's exit. Letting it start its next query at once, in one flat loop
-  // over queries and entries, was measured 0.64x as fast (strided queries)
-  // and 0.55x (the warp's lanes taking one contiguous range in order): the
-  // lanes then sit at different steps of the method, and each iteration
-  // runs the descent, expansion and output paths one after another.
+  // start their next ones together: a lane done early waits for the others.
   const uint32_t n32 = (uint32_t)nq;
-  for (uint32_t i = blockIdx.x * THREADS + threadIdx.x; i < n32; i += gridDim.x * THREADS) {
+  for (uint32_t i0 = blockIdx.x * THREADS + 32u * warp; i0 < n32; i0 += gridDim.x * THREADS) {
+    const uint32_t i = i0 + lane;
+    bool live = i < n32;
     // queries and their order are read once: streaming loads
-    const int32_t qi = perm ? __ldcs(perm + i) : (int32_t)i;
-    const float* qp = q + (int64_t)qi * q_stride;
-    const float qx = __ldcs(qp), qy = __ldcs(qp + 1), qz = __ldcs(qp + 2);
-    const int m = mq ? __ldg(mq + qi) : m_scalar;
-    if (m < 1 || m > C.n) {
-      for (int p = 0; p < k; ++p) {
-        out_idx[(int64_t)qi * k + p] = -1;
-        out_d2[(int64_t)qi * k + p] = __int_as_float(0x7f800000);
+    int32_t qi = 0;
+    float qx = 0.f, qy = 0.f, qz = 0.f;
+    int m = 0;
+    if (live) {
+      qi = perm ? __ldcs(perm + i) : (int32_t)i;
+      const float* qp = q + (int64_t)qi * q_stride;
+      qx = __ldcs(qp);
+      qy = __ldcs(qp + 1);
+      qz = __ldcs(qp + 2);
+      m = mq ? __ldg(mq + qi) : m_scalar;
+      if (m < 1 || m > C.n) {
+        live = false;
+        for (int p = 0; p < k; ++p) {
+          out_idx[(int64_t)qi * k + p] = -1;
+          out_d2[(int64_t)qi * k + p] = __int_as_float(0x7f800000);
+        }
+        atomicOr(err, 1);
       }
-      atomicOr(err, 1);
-      continue;
     }
-    bool done;
+    __syncwarp();
+    bool gave_up;
     if constexpr (LK == 8)
-      done = knn_query_smem<SortedList<8, 1, true>, DEFER>(C, qx, qy, qz, k, m, col, 8, out_idx,
-                                                            out_d2, qi);
+      gave_up = knn_query_smem<PermList<8>, DEFER>(C, live, qx, qy, qz, k, m, col, out_idx,
+                                                   out_d2, qi);
     else if constexpr (LK == 16)
-      done = knn_query_smem<PermList16, DEFER>(C, qx, qy, qz, k, m, col, 16, out_idx, out_d2, qi);
+      gave_up = knn_query_smem<PermList<16>, DEFER>(C, live, qx, qy, qz, k, m, col, out_idx,
+                                                    out_d2, qi);
     else
-      done = knn_query_smem<SortedList<32 * W, W, false>, DEFER>(C, qx, qy, qz, k, m, col, k,
-                                                                 out_idx, out_d2, qi);
+      gave_up = knn_query_smem<SortedList<32 * W, W>, DEFER>(C, live, qx, qy, qz, k, m, col,
+                                                             out_idx, out_d2, qi);
     if constexpr (DEFER) {
-      if (!done) defer[atomicAdd(ndefer, 1)] = qi;
+      if (gave_up) defer[atomicAdd(ndefer, 1)] = qi;
     }
+    __syncwarp();
   }
 }
 

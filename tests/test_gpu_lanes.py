@@ -1,0 +1,58 @@
+"""The one-lane kernel's warps against the register-list kernel, bit for bit."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import workloads as W
+from paper_2605_02224_gb300 import Cloud
+from paper_2605_02224_gb300 import mknn as M
+from tests import parity
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def cloud():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    P, _ = W.torus(3000, 71)
+    order = W.permutation(3000, 72)
+    c = Cloud.build(P, order).upload()
+    yield c, P[order]
+    c.close()
+
+
+# k at the edges of each list kind (8, 16, 32, 64 slots)
+@pytest.mark.parametrize("k", [1, 2, 7, 8, 9, 15, 16, 17, 31, 32, 33, 48, 49, 64])
+def test_partial_warps_and_bounds(cloud, k):
+    """Warps with 1, 31 and 32 queries, queries on sites, bounds that leave
+    fewer than k sites, rows that end at an odd or even entry, and bounds out
+    of [1, n]: the plain launch and a plan give the register kernel's rows,
+    and the padded rows of invalid bounds."""
+    import torch
+    c, P = cloud
+    for nq in (1, 31, 32, 33, 289):
+        Q = np.concatenate([W.box_queries(nq, 73 + nq, [-1.6] * 3, [1.6] * 3), P[:nq]])[:nq + nq // 2]
+        rng = np.random.default_rng(nq)
+        m = rng.integers(1, 3001, Q.shape[0]).astype(np.int32)
+        m[::5] = rng.integers(1, 2 * k + 2, m[::5].size)
+        bad = np.zeros(m.size, bool)
+        bad[3::29] = True
+        m[bad] = np.where(np.arange(bad.sum()) % 2 == 0, 0, 3001)
+        q, mt = torch.from_numpy(Q).cuda(), torch.from_numpy(m).cuda()
+        want = c.knn(q, k, mt, lanes=1, placement=1)
+        got = c.knn(q, k, mt, lanes=1, placement=2)
+        idx = torch.empty_like(want[0])
+        d2 = torch.empty_like(want[1])
+        M.mknn_knn_batch([dict(cloud=c.handle, q=q, nq=q.shape[0], k=k, m=mt, out_idx=idx,
+                               out_d2=d2)], lanes=1, item_rounds=2)
+        torch.cuda.synchronize()
+        for i, d in (got, (idx, d2)):
+            assert torch.equal(i, want[0]) and torch.equal(d, want[1])
+        assert np.all(got[0].cpu().numpy()[bad] == -1)
+        assert c.check() == (1 if bad.any() else 0)
+        good = np.nonzero(~bad)[0][:40]
+        parity.check_rows(P, Q[good], k, m[good], got[0].cpu().numpy()[good],
+                          got[1].cpu().numpy()[good])
