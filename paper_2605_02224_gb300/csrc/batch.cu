@@ -178,11 +178,11 @@ __global__ void __launch_bounds__(kThreads, S <= 2 ? 5 : (S <= 4 ? 4 : 3)) knn_b
 }
 
 // The one-lane variant: one query per thread, candidate lists in shared
-// memory, 256-thread blocks held to 48 registers as in the plain kernel.
+// memory, 256-thread blocks held to the registers of the plain kernel's.
 // LK: the list kind of the segment's class (8, 16 or 0), as in the plain
 // kernel.
 template <int THREADS, int W, int LK, bool DEFER>
-__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : 1) knn_batch_smem_kernel(const ReqDev* __restrict__ reqs,
+__global__ void __launch_bounds__(THREADS, THREADS == 256 ? (LK == 0 ? 3 : 5) : 1) knn_batch_smem_kernel(const ReqDev* __restrict__ reqs,
                                                                  const Item* __restrict__ items,
                                                                  int nitems,
                                                                  int* __restrict__ next,
@@ -199,6 +199,8 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : 1) knn_batch_sme
       serve_item_smem<PermList<8>, DEFER>(reqs[w.req], w, col);
     else if constexpr (LK == 16)
       serve_item_smem<PermList<16>, DEFER>(reqs[w.req], w, col);
+    else if constexpr (W == 1)
+      serve_item_smem<PermList32, DEFER>(reqs[w.req], w, col);
     else
       serve_item_smem<SortedList<32 * W, W>, DEFER>(reqs[w.req], w, col);
   }

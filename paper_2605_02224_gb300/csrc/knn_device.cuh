@@ -546,7 +546,9 @@ __device__ __forceinline__ void knn_query_thread(const CloudDev& C, float qx, fl
 // with no data-dependent loop where that pays.
 //  * PermList<8> (k <= 8), PermList<16> (k <= 16): keys stay where they were
 //    written, a register holds their order.
-//  * SortedList (k > 16): keys kept in position order; an insertion shifts
+//  * PermList32 (k <= 32): two such registers, for the nearer 16 and the
+//    others.
+//  * SortedList (k > 32): keys kept in position order; an insertion shifts
 //    the tail by one slot (a loop as long as the longest shift among the
 //    lanes inserting).
 __device__ __forceinline__ uint64_t pack_key(float d, uint32_t r) {
@@ -741,6 +743,86 @@ struct PermList {
     return (int)((uint32_t)key - 1u);
   }
 };
+// 17 <= k <= 32: two permutation words over 32 slots, one for the nearer 16
+// positions (near) and one for the others (far). An insertion searches one of
+// the halves; a key that drops out of the nearer one goes to the front of the
+// other. As in PermList the k positions are the last k of 32, here without
+// memory for the 32 - k unused slots: they are never read (the search takes
+// their keys as below every other). 500k mixed queries on the 1M-site torus,
+// k = 32: 2.73 ms with a sorted list and its shift loop, 2.53 ms now. What
+// bounds it is the list's 256 bytes per thread: 24 warps per SM, so the block
+// is held to three per SM and takes the registers it wants (72, no spills).
+struct PermList32 {
+  uint64_t* col;      // slot s at col[s * 32], s >= 32 - k
+  uint64_t near, far; // bits 4j..4j+3: the slot of position j (16 + j: less 16)
+  uint32_t done;      // by position
+  uint64_t worst;     // key of position 31 (a pad while fewer than k entries)
+
+  __device__ __forceinline__ void init(uint64_t* c, int k) {
+    col = c - (32 - k) * 32;
+    near = far = PermWord<16>::identity;
+    done = (1u << (32 - k)) - 1u;
+    worst = kPadKey;
+    for (int i = 0; i < k; ++i) c[i * 32] = kPadKey;
+  }
+  static __device__ __forceinline__ uint32_t slot(uint64_t perm, int sh) {
+    return (uint32_t)(perm >> sh) & 15u;
+  }
+  static __device__ __forceinline__ uint64_t opened(uint64_t perm, int sh, uint32_t w) {
+    const uint64_t low = perm & ((1ull << sh) - 1);
+    return low | ((perm ^ low) << 4) | ((uint64_t)w << sh);
+  }
+  // key of position pos (one of the last k)
+  __device__ __forceinline__ uint64_t at(int pos) const {
+    const bool f = pos >= 16;
+    return col[(slot(f ? far : near, 4 * (pos & 15)) + (f ? 16 : 0)) * 32];
+  }
+  __device__ __forceinline__ uint64_t key_at(int pos, int k) const { return at(32 - k + pos); }
+  __device__ __forceinline__ void to_far(uint64_t key) {
+    const uint32_t w = (uint32_t)(far >> 60);
+    col[(16 + w) * 32] = key;
+    far = (far << 4) | w;
+  }
+  // Inserts key c unless present; requires c < worst.
+  __device__ __forceinline__ void insert(uint64_t c, int k) {
+    const uint64_t top = col[(uint32_t)(near >> 60) * 32];  // position 15
+    const bool f = c > top;
+    const uint64_t perm = f ? far : near;
+    uint64_t* half = f ? col + 16 * 32 : col;
+    const int unused = f ? 0 : 4 * (32 - k);
+    int sh = 0;  // four times the number of the half's keys below c
+#pragma unroll
+    for (int step = 8; step >= 1; step >>= 1) {
+      const int at_sh = sh + 4 * (step - 1);
+      if (at_sh < unused || half[slot(perm, at_sh) * 32] < c) sh += 4 * step;
+    }
+    if (half[slot(perm, sh) * 32] == c) return;
+    const uint32_t w = (uint32_t)(perm >> 60);
+    const uint64_t opn = opened(perm, sh, w);
+    half[w * 32] = c;
+    if (f) {
+      far = opn;
+    } else {
+      near = opn;
+      to_far(top);
+    }
+    const uint32_t fl = done & ((1u << ((sh >> 2) + (f ? 16 : 0))) - 1u);
+    done = fl | ((done ^ fl) << 1);
+    worst = col[(16 + (uint32_t)(far >> 60)) * 32];
+  }
+  __device__ __forceinline__ int next(int) {
+    const uint32_t c = ~done & 0x7fffffffu;
+    if (c == 0u) return -1;
+    const int pos = __ffs((int)c) - 1;
+    const uint64_t key = at(pos);
+    if (key == kPadKey) return -1;  // pads only from here on
+    done |= 1u << pos;
+    return (int)((uint32_t)key - 1u);
+  }
+};
+__device__ __forceinline__ uint64_t list_key(const PermList32& N, int p, int k) {
+  return N.key_at(p, k);
+}
 template <int KS, int W>
 __device__ __forceinline__ uint64_t list_key(const SortedList<KS, W>& N, int p, int) {
   return N.key_at(p);
@@ -861,12 +943,12 @@ __device__ __forceinline__ bool knn_query_smem(const CloudDev& C, bool live, flo
       }
     }
     end = rr.y;
-    skip = rr.x & 1;
-    e = rr.x - skip;
+    e = rr.x & ~1;
     open = -1;
     ev = kRowEnd;
     if (rr.x < end) {
       load_pair(C.ent + e, a, b);
+      skip = rr.x & 1;
       ev = 0u;
     }
   };
@@ -883,8 +965,8 @@ __device__ __forceinline__ bool knn_query_smem(const CloudDev& C, bool live, flo
         s1 = __float_as_int(b.w);
         const bool more = e + 2 < end && s1 < m;
         if (!skip && s0 < m && !(d0 > thr)) ev = kHit0;
-        if (e + 1 < end && s1 < m && !(d1 > thr)) ev |= kHit1;
         skip = 0;
+        if (e + 1 < end && s1 < m && !(d1 > thr)) ev |= kHit1;
         if (more) {
           e += 2;
           load_pair(C.ent + e, a, b);

@@ -112,13 +112,14 @@ cudaError_t run_thread(const CloudDevHost& c, const PlainLaunch& L, cudaStream_t
 // warp w owns column l of the warp's [kcap][32] keys). 256-thread blocks are
 // held to 48 registers (five blocks per SM, no spills): left alone the
 // compiler picks either 40 registers with spills or 64, both measured
-// 5%-20% slower, and 4 or 6 blocks per SM were slower too.
+// 5%-20% slower, and 4 or 6 blocks per SM were slower too (the torus batch at
+// k = 16: 6.45 ms with 4; 1M bumpy queries at k = 4: 0.62 ms with 4, 0.59 ms
+// with 6, 0.57 ms with 5). Lists of 32 slots leave room for three blocks.
 // LK: the list kind (8: PermList<8>, k <= 8; 16: PermList<16>, 9 <= k <= 16;
-// 0: SortedList of k slots searched over 32 W). DEFER (a
-// cloud with box trees): a query that gives up (knn_query_smem) is appended
+// 0: PermList32, k <= 32, or SortedList searched over 32 W). DEFER (a cloud with box trees): a query that gives up (knn_query_smem) is appended
 // to defer[0 .. *ndefer) for the one-warp kernel.
 template <int THREADS, int W, int LK, bool DEFER>
-__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : 1) knn_plain_smem_kernel(
+__global__ void __launch_bounds__(THREADS, THREADS == 256 ? (LK == 0 ? 3 : 5) : 1) knn_plain_smem_kernel(
     CloudDev C, const float* __restrict__ q, int q_stride, int64_t nq, int k, int kcap,
     const int32_t* __restrict__ mq, int m_scalar, const int32_t* __restrict__ perm,
     int32_t* __restrict__ out_idx, float* __restrict__ out_d2, int32_t* __restrict__ err,
@@ -162,6 +163,9 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 5 : 1) knn_plain_sme
     else if constexpr (LK == 16)
       gave_up = knn_query_smem<PermList<16>, DEFER>(C, live, qx, qy, qz, k, m, col, out_idx,
                                                     out_d2, qi);
+    else if constexpr (W == 1)
+      gave_up = knn_query_smem<PermList32, DEFER>(C, live, qx, qy, qz, k, m, col, out_idx, out_d2,
+                                                  qi);
     else
       gave_up = knn_query_smem<SortedList<32 * W, W>, DEFER>(C, live, qx, qy, qz, k, m, col,
                                                              out_idx, out_d2, qi);
