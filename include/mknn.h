@@ -211,8 +211,8 @@ mknn_status mknn_cloud_load(const char* path, mknn_cloud** out);
 /* ------------------------------------------------------------------ query
  * mknn_knn: exact k-NN for a batch of queries (Algorithms 1 and 2, with the
  * prefix bound of Sec. 4.2): one query per GPU thread with its candidate
- * list in shared memory, or a group of lanes per query on clouds with very
- * long successor lists and for launches too small to fill the GPU.
+ * list in shared memory, or one warp per query from k = 48 up and in small
+ * launches.
  *   cloud     uploaded cloud.
  *   q         device float32, nq rows of q_stride floats (x, y, z first).
  *   nq        number of queries, 0 <= nq < 2^31 - 1.
@@ -234,10 +234,11 @@ mknn_status mknn_knn(const mknn_cloud* cloud, const float* q, int64_t nq, int32_
 
 /* Tuning knobs of one query launch; zero-initialise for defaults. */
 typedef struct {
-  int32_t lanes;        /* lanes per query: 0 = default (1, or 32 from
-                           k = 48 up, or more for small batches and
-                           clouds with very long successor lists - for
-                           k > 8 when the cloud has box trees), or
+  int32_t lanes;        /* lanes per query: 0 = default (32 from k = 48
+                           up, in batches below about 32,768 + 896 k
+                           queries - 2.5 times that on clouds with long
+                           successor lists - and on clouds with very
+                           long lists and no box trees; else 1), or
                            1, 4, 8, 16, 32 (4 and 8 hold k <= 64; one
                            lane above 64 needs placement 2 and no
                            counters) */
@@ -424,8 +425,8 @@ mknn_status mknn_knn_batch(const mknn_batch_req* reqs, int32_t nreq, const mknn_
  * warm-up) on max(sample, 2 x SMs x 2048) queries of that request (tiled
  * when it has fewer); the fastest (lanes, placement) goes into the
  * process-wide tuning table. Plans, plain launches and the server take the
- * table's entry, widened to more lanes when a launch is too small to fill
- * the GPU one query per thread. If the environment variable MKNN_TUNE_LOG
+ * table's entry, one warp per query where it says one lane and the launch is
+ * too small for that. If the environment variable MKNN_TUNE_LOG
  * names a file, one line per timed candidate (k, n, hub bucket, sample,
  * lanes, placement, ms) is appended to it. Synchronises the stream.
  * Errors: EINVAL, ENOMEM, ECUDA. */

@@ -301,48 +301,41 @@ int nbucket_of(int64_t n) {
   return b;
 }
 
-// Untuned default: one query per thread, except on clouds with hub rows
-// (a successor list of 2^12 entries or more, typical of nearly coplanar
-// sites), where a whole warp per query scans the long rows 32 entries at a
-// time. Timed on 64 mixed clouds, 32 lanes won on 16 of the 17 hub clouds
-// (by 1.2x-3.9x) and lost on all but one of the others (by up to 20x).
-// With box trees and the hand-over of mknn_knn_ex (one lane per query,
-// the queries that meet a list with a tree answered by the one-warp kernel)
-// one lane is the default up to k = 8: on the 20 patch clouds of that mix
-// with trees it took 119 ms against 124 ms for 32 lanes, winning at k <= 8
-// on all but two and losing at k = 16 and 32 by up to 1.7x.
+// Untuned default on a cloud whose long lists have no trees (a dynamic
+// cloud): with a successor list of 2^12 entries or more, a whole warp per
+// query, which scans the long rows 32 entries at a time.
 constexpr int kHubBucketWide = 12;
-constexpr int kHandoverMaxK = 8;
-int heuristic_lanes(int k, int hub, bool handover) {
-  if (handover && k <= kHandoverMaxK) return default_lanes(k);
-  return hub >= kHubBucketWide ? 32 : default_lanes(k);
+
+// Queries of one launch from which one lane per query is faster than one
+// warp per query. One lane per query takes about the time of its longest
+// query whatever the number of queries, until they fill the GPU; one warp
+// per query takes time in proportion to it. On a 300k-site torus (queries
+// half in the box, half near the surface; us for one lane / one warp per
+// query at 30,000 and 60,000 queries, the locality sort included):
+//   k = 1: 98 / 93, 99 / 147     k = 8: 185 / 146, 189 / 247
+//   k = 16: 274 / 208, 291 / 357   k = 32: 501 / 312, 532 / 547
+// and on a 200k-site patch cloud with trees, at 60,000 and 200,000 queries:
+//   k = 1: 250 / 174, 341 / 479   k = 8: 438 / 291, 639 / 828
+//   k = 16: 643 / 429, 989 / 1282   k = 32: 1024 / 687, 1901 / 2090
+// A lane that scans a list of hundreds of entries takes as long as one that
+// gives up at a tree (12k-site patch cloud, longest list 757, no trees: k = 4
+// 340 / 157, 371 / 430), so such clouds take the second line too.
+// Register groups of 4, 8 and 16 lanes are slower than both at every size
+// (100,000 queries, k = 16: 1,638 / 994 / 837 us against 320), so the rule
+// never takes them.
+constexpr int kHubBucketLong = 9;  // a list of 2^9 - 1 entries or more
+int64_t one_lane_min_queries(int k, int hub, bool trees) {
+  const int64_t q = 32768 + 896 * (int64_t)k;
+  return (trees || hub >= kHubBucketLong) ? q * 5 / 2 : q;
 }
 
 }  // namespace
 
-int fill_lanes(int64_t nq, int k) {
-  // One query per thread fills the GPU with (SMs x resident threads)
-  // queries; resident threads of the shared-memory variant are limited by
-  // its 48 registers (1280 per SM) and by 8 k bytes of list per thread.
-  // Smaller batches give each query a group of lanes so all SMs work.
-  const int64_t per_sm = std::min<int64_t>(1280, 233472 / (8 * (int64_t)std::max(k, 8)));
-  const int64_t target = (int64_t)num_sms() * per_sm;
-  int lanes = 1;
-  while (lanes < 32 && nq * lanes < target) lanes <<= 1;
-  if (lanes == 2) lanes = 4;  // no two-lane variant
-  return lanes;
-}
-
 Mode choose_mode(int k, int64_t n, int hub, int64_t nq, bool trees) {
   const Mode t = tuned_mode(k, n, hub);
-  const int fill = fill_lanes(nq, k);
-  // one lane with the hand-over only where the launch stays one lane wide
-  const int base = t.lanes ? t.lanes : heuristic_lanes(k, hub, trees && fill == 1);
-  int lanes = std::max(base, fill);
-  // widened on a cloud with box trees: the one-warp kernel, which walks them
-  // (register groups would read the long lists through)
-  if (trees && lanes > base && lanes < 32) lanes = 32;
-  while (lanes < 32 && variant_index(lanes, k, 1) < 0) lanes <<= 1;  // e.g. 4 lanes hold k <= 16
+  const int wide = (hub >= kHubBucketWide && !trees) ? 32 : default_lanes(k);
+  int lanes = t.lanes ? t.lanes : wide;
+  if (lanes == 1 && nq < one_lane_min_queries(k, hub, trees)) lanes = 32;
   const int placement = (t.lanes && lanes == t.lanes) ? t.placement : default_placement(k, lanes);
   return Mode{lanes, placement};
 }

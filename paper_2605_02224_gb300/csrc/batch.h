@@ -155,14 +155,10 @@ cudaError_t launch_segments(const ReqDev* d_reqs, const Item* d_items, int* d_ne
 Mode tuned_mode(int k, int64_t n, int hub);
 void set_tuned_mode(int k, int64_t n, int hub, Mode m);
 // Mode for a launch of nq queries: the tuned (or default) lanes for
-// (k, n, hub), widened for batches too small to fill the GPU one query per
-// thread, and the tuned placement (or the default for those lanes).
+// (k, n, hub) and their placement; one lane per query turns into one warp
+// per query in a launch too small for it.
 // trees: the cloud has box trees and the launch can use them (the one-warp
-// kernel walks them; one lane hands queries that meet them over to it):
-// then one lane is the default for small k when the launch stays one lane
-// wide, and a launch widened for its size goes to 32 lanes.
+// kernel walks them; one lane hands queries that meet them over to it).
 Mode choose_mode(int k, int64_t n, int hub, int64_t nq, bool trees = false);
-// The smallest lane width that fills the GPU with nq queries of this k.
-int fill_lanes(int64_t nq, int k);
 
 }  // namespace mknn

@@ -56,3 +56,32 @@ def test_partial_warps_and_bounds(cloud, k):
         good = np.nonzero(~bad)[0][:40]
         parity.check_rows(P, Q[good], k, m[good], got[0].cpu().numpy()[good],
                           got[1].cpu().numpy()[good])
+
+
+@pytest.mark.parametrize("surface,n", [("torus", 4000), ("patches", 12000), ("patches", 90000)])
+@pytest.mark.parametrize("k", [1, 16, 32, 47, 48])
+def test_default_lanes_around_the_crossover(surface, n, k):
+    """Launches just below and above the number of queries from which one
+    lane per query is the default, on clouds without long lists, with them,
+    and with box trees: the plain launch, the no-allocation one and a plan
+    give the rows of one lane and of one warp per query."""
+    import torch
+    P, _ = W.surface(surface, n, 81)
+    order = W.permutation(n, 82)
+    c = Cloud.build(P, order).upload()
+    lo, hi = W.padded_box(P)
+    base = 32768 + 896 * k
+    for nq in (base - 1, base, base * 5 // 2 - 1, base * 5 // 2):
+        q = torch.from_numpy(W.box_queries(nq, 83, lo, hi)).cuda()
+        want = c.knn(q, k, lanes=32, placement=2)
+        runs = [c.knn(q, k), c.knn(q, k, lanes=1, placement=2)]
+        for call in (lambda i, d: M.mknn_knn_noalloc(c.handle, q, nq, 3, k, None, 0, i, d),
+                     lambda i, d: M.mknn_knn_batch([dict(cloud=c.handle, q=q, nq=nq, k=k,
+                                                         out_idx=i, out_d2=d)])):
+            idx, d2 = torch.full_like(want[0], -9), torch.full_like(want[1], -9)
+            call(idx, d2)
+            runs.append((idx, d2))
+        torch.cuda.synchronize()
+        for i, d in runs:
+            assert torch.equal(i, want[0]) and torch.equal(d, want[1])
+    c.close()
