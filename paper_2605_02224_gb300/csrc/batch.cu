@@ -11,7 +11,7 @@
 // item with one atomic. Items of one request are contiguous in a queue, so
 // the warps working at any moment share one cloud's table in L2; requests
 // are queued by decreasing estimated cost so that a queue ends with short
-// items. The one-lane launch and the group launches run on two streams.
+// items. The segments of a small plan run side by side on a few streams.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -466,7 +466,7 @@ std::vector<Segment> make_segments(std::vector<Item>& items, int blocks_per_sm,
     return slots <= 8 ? 0 : (slots <= 16 ? 1 : (slots <= 32 ? 2 : 3));
   };
   std::stable_sort(items.begin(), items.end(), [&](const Item& a, const Item& c) {
-    return rank(a.variant) != rank(c.variant) ? rank(a.variant) < rank(c.variant) : cls(a) < cls(c);
+    return rank(a.variant) != rank(c.variant) ? rank(a.variant) < rank(c.variant) : cls(a) > cls(c);
   });
   std::vector<Segment> segs;
   for (int i = 0; i < (int)items.size();) {
@@ -510,25 +510,44 @@ cudaError_t launch_handover(const ReqDev* d_reqs, Handover* d_ho, int c, int gri
                           0, s);
 }
 
-cudaError_t launch_segments(const ReqDev* d_reqs, const Item* d_items, int* d_next,
-                            const std::vector<Segment>& segs, cudaStream_t s, cudaStream_t aux,
-                            cudaEvent_t fork, cudaEvent_t join, int64_t queries) {
-  bool one = false, group = false;
-  for (const Segment& g : segs) (is_smem_variant(g.launch.variant) ? one : group) = true;
-  const bool split = one && group && aux && queries <= kSplitMaxQueries;
-  cudaError_t e = cudaSuccess;
-  if (split) {
-    if ((e = cudaEventRecord(fork, s)) != cudaSuccess) return e;
-    if ((e = cudaStreamWaitEvent(aux, fork, 0)) != cudaSuccess) return e;
+bool SideStreams::create() {
+  bool ok = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming) == cudaSuccess;
+  for (int i = 0; i < kSideStreams && ok; ++i)
+    ok = cudaStreamCreateWithFlags(&s[i], cudaStreamNonBlocking) == cudaSuccess &&
+         cudaEventCreateWithFlags(&join[i], cudaEventDisableTiming) == cudaSuccess;
+  if (!ok) cudaGetLastError();
+  return ok;
+}
+
+void SideStreams::destroy() {
+  if (fork) cudaEventDestroy(fork);
+  for (int i = 0; i < kSideStreams; ++i) {
+    if (join[i]) cudaEventDestroy(join[i]);
+    if (s[i]) cudaStreamDestroy(s[i]);
   }
+  *this = SideStreams{};
+}
+
+cudaError_t launch_segments(const ReqDev* d_reqs, const Item* d_items, int* d_next,
+                            const std::vector<Segment>& segs, cudaStream_t s,
+                            const SideStreams& side, int64_t queries) {
+  const bool split = segs.size() > 1 && side.fork && queries <= kSplitMaxQueries;
+  const int nside = split ? (int)std::min<size_t>(kSideStreams, segs.size() - 1) : 0;
+  cudaError_t e = cudaSuccess;
+  if (split && (e = cudaEventRecord(side.fork, s)) != cudaSuccess) return e;
+  for (int i = 0; i < nside; ++i)
+    if ((e = cudaStreamWaitEvent(side.s[i], side.fork, 0)) != cudaSuccess) return e;
   for (size_t i = 0; i < segs.size() && e == cudaSuccess; ++i) {
     const Segment& g = segs[i];
-    cudaStream_t st = (split && !is_smem_variant(g.launch.variant)) ? aux : s;
-    e = launch_batch_kernel(d_reqs, d_items + g.begin, g.count, d_next + i, g.launch, st);
+    const int on = (int)(i % (size_t)(nside + 1));
+    e = launch_batch_kernel(d_reqs, d_items + g.begin, g.count, d_next + i, g.launch,
+                            on ? side.s[on - 1] : s);
   }
-  if (e != cudaSuccess || !split) return e;
-  if ((e = cudaEventRecord(join, aux)) != cudaSuccess) return e;
-  return cudaStreamWaitEvent(s, join, 0);
+  for (int i = 0; i < nside && e == cudaSuccess; ++i) {
+    if ((e = cudaEventRecord(side.join[i], side.s[i])) != cudaSuccess) return e;
+    e = cudaStreamWaitEvent(s, side.join[i], 0);
+  }
+  return e;
 }
 
 Mode tuned_mode(int k, int64_t n, int hub) {
@@ -562,8 +581,7 @@ struct mknn_batch {
   void* d_ws = nullptr;          // sort scratch: shared histogram, per-request cells and orders
   size_t ws_bytes = 0;
   std::vector<size_t> cell_off, perm_off;  // per request, 0 if not sorted
-  cudaStream_t aux = nullptr;    // second branch: the group segments
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  SideStreams side;              // segments of a small plan run side by side
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   int64_t total_queries = 0;
@@ -592,9 +610,7 @@ void free_plan(mknn_batch* b) {
   cudaFree(b->d_ws);
   cudaFree(b->d_ho);
   cudaFree(b->d_ho_pairs);
-  if (b->ev_fork) cudaEventDestroy(b->ev_fork);
-  if (b->ev_join) cudaEventDestroy(b->ev_join);
-  if (b->aux) cudaStreamDestroy(b->aux);
+  b->side.destroy();
   delete b;
 }
 
@@ -618,8 +634,7 @@ cudaError_t enqueue(mknn_batch* b, cudaStream_t s) {
                                 (int32_t*)((char*)b->d_ws + b->perm_off[r]), s);
     if (e != cudaSuccess) return e;
   }
-  e = launch_segments(b->d_reqs, b->d_items, b->d_next, b->segs, s, b->aux, b->ev_fork,
-                      b->ev_join, b->total_queries);
+  e = launch_segments(b->d_reqs, b->d_items, b->d_next, b->segs, s, b->side, b->total_queries);
   for (int c = 0; c < 3 && e == cudaSuccess; ++c)
     if (b->ho_class[c]) e = launch_handover(b->d_reqs, b->d_ho, c, b->ho_grid[c], s);
   return e;
@@ -768,16 +783,10 @@ mknn_status mknn_batch_create(const mknn_batch_req* reqs, int32_t nreq,
     free_plan(raw);
     return bfail(MKNN_ECUDA, std::string("plan upload: ") + cudaGetErrorString(e));
   }
-  bool one = false, group = false;
-  for (const Segment& g : b->segs) (is_smem_variant(g.launch.variant) ? one : group) = true;
-  if (one && group) {
-    if ((e = cudaStreamCreateWithFlags(&b->aux, cudaStreamNonBlocking)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming)) != cudaSuccess) {
-      mknn_batch* raw = b.release();
-      free_plan(raw);
-      return bfail(MKNN_ECUDA, std::string("plan streams: ") + cudaGetErrorString(e));
-    }
+  if (b->segs.size() > 1 && b->total_queries <= kSplitMaxQueries && !b->side.create()) {
+    mknn_batch* raw = b.release();
+    free_plan(raw);
+    return bfail(MKNN_ECUDA, "plan streams");
   }
   if (o.graph >= 0) {
     cudaStream_t cs;

@@ -127,27 +127,34 @@ struct Segment {
   int begin = 0, count = 0;
   BatchLaunch launch;
 };
-// Reorders items by variant (the one-lane kernels' first, each variant's
-// items in their given order) and returns one segment per variant present;
+// Reorders items by variant (the one-lane kernels' first, larger lists
+// before smaller; each class's items in their given order) and returns one segment per variant present;
 // req_k[r] is request r's k (a one-lane segment's list capacity is its
 // largest k).
 std::vector<Segment> make_segments(std::vector<Item>& items, int blocks_per_sm,
                                    const std::vector<int>& req_k);
+// Streams beside a launch's own for its segments, and the events that fork
+// and join them.
+constexpr int kSideStreams = 3;
+struct SideStreams {
+  cudaStream_t s[kSideStreams] = {};
+  cudaEvent_t fork = nullptr, join[kSideStreams] = {};
+  bool create();   // false when the driver refuses; destroy() is still due
+  void destroy();
+};
 // Launches every segment, segment i draining the queue counter d_next[i]
-// (zero on entry). With one-lane and group segments both present in a
-// launch of at most kSplitMaxQueries queries, the group segments run one
-// after another on `aux`, forked from s and joined back, concurrently with
-// the one-lane segments on s; otherwise all run on s in order. Two
-// persistent launches that each size their grid for the whole GPU fill
-// each other's tails in a small launch, and share the GPU worse than they
-// run in turn in a large one: the 64-cloud batching plan (57.6M queries)
-// took 224 ms in turn against 234 ms on two streams, while the serving
-// loop (packs of at most 2^17 queries) saturated at 6,510 requests/s on
-// two streams against 5,717 in turn.
+// (zero on entry). The segments of a launch of at most kSplitMaxQueries
+// queries are spread over s and the side streams (forked from s and joined
+// back); otherwise all run on s in order. Persistent launches that each size
+// their grid for the whole GPU fill each other's tails in a small launch,
+// and share the GPU worse than they run in turn in a large one: the 64-cloud
+// batching plan (57.6M queries) took 224 ms in turn against 234 ms on two
+// streams, the plan of 12 clouds (0.76M queries, three one-lane segments)
+// 4.22 ms in turn and 3.30 side by side, the larger lists first.
 constexpr int64_t kSplitMaxQueries = int64_t(1) << 21;
 cudaError_t launch_segments(const ReqDev* d_reqs, const Item* d_items, int* d_next,
-                            const std::vector<Segment>& segs, cudaStream_t s, cudaStream_t aux,
-                            cudaEvent_t fork, cudaEvent_t join, int64_t queries);
+                            const std::vector<Segment>& segs, cudaStream_t s,
+                            const SideStreams& side, int64_t queries);
 
 // Mode recorded by the tuner for (k, n, hub), lanes 0 if none. The tuning
 // table is keyed by k, floor(log2 n) and the cloud's hub bucket

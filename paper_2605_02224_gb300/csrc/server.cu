@@ -104,8 +104,7 @@ struct ReqRec {
 
 struct Slot {
   cudaStream_t s = nullptr;
-  cudaStream_t aux = nullptr;    // second branch for packs with both kernel families
-  cudaEvent_t fork = nullptr, join = nullptr;
+  SideStreams side;              // a pack's segments run side by side
   cudaEvent_t done = nullptr;
   // phase marks of the current launch (timing events): start, after the
   // host-to-device copies, after the kernels; `done` follows the copies back
@@ -338,11 +337,11 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
                                     (int32_t*)(dbase + R.perm_off), s);
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(d_next, 0, segs.size() * sizeof(int), s);
-    // the one-lane kernel on the slot's stream, the group kernels on its
-    // second stream, joined before the copies back
+    // the segments on the slot's stream and its side streams, joined before
+    // the copies back
     if (e == cudaSuccess)
       e = launch_segments((const ReqDev*)(dbase + reqs_off), (const Item*)(dbase + items_off),
-                          d_next, segs, s, sl.aux, sl.fork, sl.join, pack_nq);
+                          d_next, segs, s, sl.side, pack_nq);
     // the handed-over queries, after every segment
     for (int c = 0; c < 3 && handover && e == cudaSuccess; ++c)
       if (ho_cap[c] > 0)
@@ -480,9 +479,7 @@ mknn_status mknn_server_create(const mknn_server_opts* opts, mknn_server** out) 
   s->slots.resize(s->o.slots);
   for (Slot& sl : s->slots) {
     if (cudaStreamCreateWithFlags(&sl.s, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaStreamCreateWithFlags(&sl.aux, cudaStreamNonBlocking) != cudaSuccess ||
-        cudaEventCreateWithFlags(&sl.fork, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreateWithFlags(&sl.join, cudaEventDisableTiming) != cudaSuccess ||
+        !sl.side.create() ||
         cudaEventCreate(&sl.done) != cudaSuccess || cudaEventCreate(&sl.t0) != cudaSuccess ||
         cudaEventCreate(&sl.t_h2d) != cudaSuccess || cudaEventCreate(&sl.t_kern) != cudaSuccess) {
       cudaGetLastError();
@@ -635,15 +632,13 @@ mknn_status mknn_server_destroy(mknn_server* s, double timeout_s) {
   s->th.join();
   for (Slot& sl : s->slots) {
     cudaStreamSynchronize(sl.s);
-    cudaStreamSynchronize(sl.aux);
+    for (cudaStream_t a : sl.side.s) cudaStreamSynchronize(a);
     cudaEventDestroy(sl.done);
-    cudaEventDestroy(sl.fork);
-    cudaEventDestroy(sl.join);
     cudaEventDestroy(sl.t0);
     cudaEventDestroy(sl.t_h2d);
     cudaEventDestroy(sl.t_kern);
     cudaStreamDestroy(sl.s);
-    cudaStreamDestroy(sl.aux);
+    sl.side.destroy();
   }
   for (mknn_cloud* c : s->clouds) c->holders--;
   cudaFree(s->d_arena);
