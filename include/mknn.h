@@ -122,7 +122,7 @@ mknn_status mknn_cloud_from_table(const float* xyz_ranked, int64_t n, const int6
  * 24 n + 20 E plus a few words of status (a dynamic cloud also reserves
  * room for appends: a quarter more sites and entries, at least 4096 sites
  * and 65536 entries). A cloud without appends whose longest successor list
- * has 4096 entries or more also gets a box tree over every list of 256
+ * has 1024 entries or more also gets a box tree over every list of 256
  * entries or more (an index for the one-warp
  * query kernel, which searches such a list through its tree instead of
  * reading it in rank order, with the same result; Algorithms 1-2 need
@@ -178,7 +178,7 @@ mknn_status mknn_cloud_info(const mknn_cloud* cloud, int64_t* n, int64_t* E, siz
 
 /* Box trees of the device copy (mknn_cloud_upload): number of trees and
  * the entries of the lists they cover (0 and 0 before upload, for a cloud
- * built for appends, and when no list has 4096 entries). Either output may
+ * built for appends, and when no list has 1024 entries). Either output may
  * be NULL. The paper has no such index: it reads every list in rank order. */
 mknn_status mknn_cloud_trees(const mknn_cloud* cloud, int64_t* trees, int64_t* entries);
 

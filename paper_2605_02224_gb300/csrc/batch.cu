@@ -686,7 +686,7 @@ mknn_status mknn_batch_create(const mknn_batch_req* reqs, int32_t nreq,
     if (R.nq > 0 && (!R.q || !R.out_idx || !R.out_d2))
       return bfail(MKNN_EINVAL, "request " + std::to_string(r) + ": NULL device pointer");
     const Mode chosen =
-        choose_mode(R.k, R.cloud->n, R.cloud->hub_bucket(), plan_nq, R.cloud->d_hub_of != nullptr);
+        choose_mode(R.k, R.cloud->n, R.cloud->hub_bucket(), plan_nq, R.cloud->trees(R.k));
     const int lanes = o.lanes ? o.lanes : chosen.lanes;
     const int placement = o.placement ? o.placement
                                       : (o.lanes ? default_placement(R.k, lanes) : chosen.placement);
@@ -694,7 +694,7 @@ mknn_status mknn_batch_create(const mknn_batch_req* reqs, int32_t nreq,
       return bfail(MKNN_EINVAL, "request " + std::to_string(r) + ": lanes/k combination");
     b->lanes[r] = lanes;
     b->placement[r] = placement;
-    const CloudDevHost cd = R.cloud->dev();
+    const CloudDevHost cd = R.cloud->dev(R.k);
     rd[r] = ReqDev{(const float4*)cd.pts, cd.rows,   cd.succ, cd.n,  R.q_stride,
                    R.q,                   R.m,       nullptr, R.out_idx,
                    R.out_d2,              R.cloud->d_err, R.k, ms, (const float4*)cd.ent,
@@ -725,7 +725,7 @@ mknn_status mknn_batch_create(const mknn_batch_req* reqs, int32_t nreq,
   int64_t ho_cap[3] = {0, 0, 0};  // queries that may be handed over, per class
   for (int r : orderq) {
     const int v = with_trees(variant_index(b->lanes[r], reqs[r].k, b->placement[r]),
-                             reqs[r].cloud->d_hub_of != nullptr, true);
+                             reqs[r].cloud->trees(reqs[r].k), true);
     if (v == kHandoverVariant || v == kHandoverVariant128) {
       ho_cap[handover_class(reqs[r].k)] += reqs[r].nq;
       b->ho_class[handover_class(reqs[r].k)] = true;
@@ -771,7 +771,7 @@ mknn_status mknn_batch_create(const mknn_batch_req* reqs, int32_t nreq,
       return bfail(MKNN_ECUDA, std::string("plan upload: ") + cudaGetErrorString(e));
     }
     for (int r = 0; r < nreq; ++r)
-      if (reqs[r].cloud->d_hub_of) rd[r].ho = b->d_ho;
+      if (rd[r].hub_of) rd[r].ho = b->d_ho;
     for (int c = 0; c < 3; ++c)
       if (b->ho_class[c]) b->ho_grid[c] = handover_grid(c);
   }

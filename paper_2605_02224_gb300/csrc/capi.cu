@@ -90,7 +90,7 @@ void free_device(mknn_cloud* c) {
   }
   c->d_hub_of = nullptr;
   c->d_hub_desc = c->d_hub_ent = c->d_hub_node = nullptr;
-  c->hub_trees = c->hub_entries = 0;
+  c->hub_trees = c->hub_entries = c->hub_longest = 0;
   c->d_pts = nullptr;
   c->d_ent = nullptr;
   c->pts_cap = c->ent_cap = c->ent_top = 0;
@@ -382,7 +382,10 @@ mknn_status mknn_cloud_upload(mknn_cloud* c, mknn_stream_t stream) {
       }
       b_hub = b_of + b_desc + b_hent + b_node;
       c->hub_trees = H.hubs();
-      for (int64_t h = 0; h < H.hubs(); ++h) c->hub_entries += H.desc[4 * h + 1];
+      for (int64_t h = 0; h < H.hubs(); ++h) {
+        c->hub_entries += H.desc[4 * h + 1];
+        c->hub_longest = std::max<int64_t>(c->hub_longest, H.desc[4 * h + 1]);
+      }
     }
   }
   c->pts_cap = pcap;
@@ -571,7 +574,7 @@ mknn_status mknn_knn_ex(const mknn_cloud* c, const float* q, int64_t nq, int32_t
   }
   if (nq == 0) return MKNN_OK;
   if (!q || !out_idx || !out_d2) return fail(MKNN_EINVAL, "NULL device pointer");
-  const Mode chosen = choose_mode(k, c->n, c->hub_bucket(), nq, c->d_hub_of != nullptr);
+  const Mode chosen = choose_mode(k, c->n, c->hub_bucket(), nq, c->trees(k));
   int lanes = (opts && opts->lanes) ? opts->lanes : chosen.lanes;
   if (lanes != 1 && lanes != 4 && lanes != 8 && lanes != 16 && lanes != 32)
     return fail(MKNN_EINVAL, "lanes must be 1, 4, 8, 16 or 32");
@@ -590,7 +593,7 @@ mknn_status mknn_knn_ex(const mknn_cloud* c, const float* q, int64_t nq, int32_t
   // queries to the one-warp kernel (one lane on a cloud with box trees)
   const size_t sort_need = (!perm && sort_enabled(opts, nq)) ? sort_workspace_bytes(nq) + perm_bytes(nq) : 0;
   const bool wants_defer =
-      c->d_hub_of && lanes == 1 && placement == 2 && !(opts && opts->counters);
+      c->trees(k) && lanes == 1 && placement == 2 && !(opts && opts->counters);
   size_t need = sort_need + (wants_defer ? defer_bytes(nq) : 0);
   void* ws = nullptr;
   if (need > 0) {
@@ -626,7 +629,7 @@ mknn_status mknn_knn_ex(const mknn_cloud* c, const float* q, int64_t nq, int32_t
   L.lanes = lanes;
   L.blocks_per_sm = opts ? opts->blocks_per_sm : 0;
   L.placement = placement;
-  cudaError_t e = launch_knn_plain(c->dev(), L, s);
+  cudaError_t e = launch_knn_plain(c->dev(k), L, s);
   if (e != cudaSuccess) return cuda_fail(e, "knn kernel launch");
   return MKNN_OK;
 }

@@ -10,6 +10,7 @@
 #include <memory>
 
 #include "builder.h"
+#include "hub_index.h"
 #include "knn_kernels.h"
 
 struct mknn_cloud {
@@ -42,6 +43,7 @@ struct mknn_cloud {
   void* d_hub_ent = nullptr;     // float4 per entry
   void* d_hub_node = nullptr;    // two float4 per node
   int64_t hub_trees = 0, hub_entries = 0;  // trees, and the entries of their lists
+  int64_t hub_longest = 0;                 // the longest of these lists
   size_t dev_bytes = 0;
   // device capacities: sites (d_pts, d_rows) and entries (d_succ, d_ent);
   // a dynamic cloud's rows live in an append-only arena: row i occupies
@@ -76,16 +78,23 @@ struct mknn_cloud {
     return hb;
   }
   mutable std::atomic<int> hub_{-1};
-  mknn::CloudDevHost dev() const {
+  // Does a launch of this k use the cloud's box trees?
+  bool trees(int k) const {
+    return d_hub_of && (k < mknn::kWarpMinK || hub_longest >= mknn::kHubMinLongestWarp);
+  }
+  // The device copy as a launch of this k reads it (any k: with its trees).
+  mknn::CloudDevHost dev(int k = 0) const {
     mknn::CloudDevHost c;
     c.pts = d_pts;
     c.rows = d_rows;
     c.succ = d_succ;
     c.ent = d_ent;
-    c.hub_of = d_hub_of;
-    c.hub_desc = d_hub_desc;
-    c.hub_ent = d_hub_ent;
-    c.hub_node = d_hub_node;
+    if (trees(k)) {
+      c.hub_of = d_hub_of;
+      c.hub_desc = d_hub_desc;
+      c.hub_ent = d_hub_ent;
+      c.hub_node = d_hub_node;
+    }
     c.n = (int32_t)n;
     for (int i = 0; i < 3; ++i) {
       c.lo[i] = lo[i];

@@ -25,13 +25,22 @@
 namespace mknn {
 
 // Lists at least this long get a box tree, in a cloud whose longest list
-// has at least kHubMinLongest entries. The walk's code slows the one-warp
-// kernel's scan of the other lists by about a quarter (registers), which
-// only clouds with real hubs win back: on the 1M-site torus (longest list
-// 389) trees made k = 100 queries 28% slower; on 1.3M-site patch clouds
-// (longest lists 10^5) 4.8x faster.
+// has at least kHubMinLongest entries. A query that reads such a list
+// through holds up its warp, and with few queries the launch: on the
+// 20k-site patch cloud (longest list 2,695; us without / with trees, 200,000
+// queries) k = 4 717 / 289, k = 16 1262 / 680, k = 32 1731 / 1448, and the
+// plan of 12 clouds, two of them such clouds, 3.30 / 1.64 ms. Below, they
+// give less than they cost (5k sites, longest list 563: k = 16 556 / 502,
+// k = 32 931 / 1111).
 constexpr int64_t kHubMinRow = 256;
-constexpr int64_t kHubMinLongest = 4096;
+constexpr int64_t kHubMinLongest = 1024;
+// From this longest list on the trees serve launches with one warp per query
+// by default (k >= 48) too. The walk's code slows the one-warp kernel's scan
+// of the other lists by 15-28% (registers), which shorter lists don't win
+// back: 200,000 queries at k = 64, 20k-site patch cloud, 3,980 us without and
+// 4,568 with trees; on 1.3M-site patch clouds (longest lists 10^5) trees are
+// 4.8x faster.
+constexpr int64_t kHubMinLongestWarp = 4096;
 // Levels of a tree: 32^4 chunks of 32 entries at most; longer lists are
 // scanned in rank order.
 constexpr int kHubMaxLevels = 4;

@@ -126,7 +126,7 @@ extern "C" mknn_status mknn_knn_noalloc(const mknn_cloud* c, const float* q, int
     return MKNN_EINVAL;
   }
   cudaStream_t s = (cudaStream_t)stream;
-  const mknn::CloudDevHost cd = c->dev();
+  const mknn::CloudDevHost cd = c->dev(k);
   // layout: [histogram + cells (sort scratch)] [processing order]; small
   // batches skip the locality sort, as mknn_knn does
   int32_t* perm = nullptr;

@@ -267,7 +267,7 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
     for (int i = 0; i < nreq; ++i) {
       const mknn_request& q = recs[tickets[i] - 1].r;
       const mknn_cloud* c = clouds[q.cloud];
-      const Mode chosen = choose_mode(q.k, c->n, c->hub_bucket(), pack_nq, c->d_hub_of != nullptr);
+      const Mode chosen = choose_mode(q.k, c->n, c->hub_bucket(), pack_nq, c->trees(q.k));
       lanes[i] = o.lanes ? o.lanes : chosen.lanes;
       placement[i] = o.lanes ? default_placement(q.k, lanes[i]) : chosen.placement;
     }
@@ -279,7 +279,7 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
       ReqRec& R = recs[tickets[i] - 1];
       const mknn_request& q = R.r;
       const mknn_cloud* c = clouds[q.cloud];
-      const CloudDevHost cd = c->dev();
+      const CloudDevHost cd = c->dev(q.k);
       const size_t qb = (size_t)q.nq * 12;
       const void* src = q.q;
       if (!R.q_pinned) {

@@ -58,8 +58,9 @@ def test_partial_warps_and_bounds(cloud, k):
                           got[1].cpu().numpy()[good])
 
 
-@pytest.mark.parametrize("surface,n", [("torus", 4000), ("patches", 12000), ("patches", 90000)])
-@pytest.mark.parametrize("k", [1, 16, 32, 47, 48])
+@pytest.mark.parametrize("surface,n", [("torus", 4000), ("patches", 12000),
+                                       ("patches", 30000), ("patches", 90000)])
+@pytest.mark.parametrize("k", [1, 16, 32, 47, 48, 100])
 def test_default_lanes_around_the_crossover(surface, n, k):
     """Launches just below and above the number of queries from which one
     lane per query is the default, on clouds without long lists, with them,
@@ -73,7 +74,7 @@ def test_default_lanes_around_the_crossover(surface, n, k):
     base = 32768 + 896 * k
     for nq in (base - 1, base, base * 5 // 2 - 1, base * 5 // 2):
         q = torch.from_numpy(W.box_queries(nq, 83, lo, hi)).cuda()
-        want = c.knn(q, k, lanes=32, placement=2)
+        want = c.knn(q, k, lanes=32, placement=1)
         runs = [c.knn(q, k), c.knn(q, k, lanes=1, placement=2)]
         for call in (lambda i, d: M.mknn_knn_noalloc(c.handle, q, nq, 3, k, None, 0, i, d),
                      lambda i, d: M.mknn_knn_batch([dict(cloud=c.handle, q=q, nq=nq, k=k,
