@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? (LK == 0 ? 3 : 5) : 
 // warp, static): the warp takes an item and answers its queries one after
 // another.
 template <int KC, bool TREES>
-__global__ void __launch_bounds__(kThreads) knn_batch_warp_kernel(const ReqDev* __restrict__ reqs,
+__global__ void __launch_bounds__(kThreads, kWarpBlocks(KC, TREES)) knn_batch_warp_kernel(const ReqDev* __restrict__ reqs,
                                                                   const Item* __restrict__ items,
                                                                   int nitems,
                                                                   int* __restrict__ next,
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kThreads) knn_batch_warp_kernel(const ReqDev* 
 // lists of KC keys): one warp per query, the box trees walked; launched
 // after every segment, it reads the number handed over from the device.
 template <int KC>
-__global__ void __launch_bounds__(kThreads) knn_batch_handover_kernel(
+__global__ void __launch_bounds__(kThreads, kWarpBlocks(KC, true)) knn_batch_handover_kernel(
     const ReqDev* __restrict__ reqs, Handover* __restrict__ ho, int cls) {
   __shared__ uint64_t lists[kThreads / 32][kWarpListWords(KC)];
   const int warp = (int)(threadIdx.x >> 5);
@@ -311,22 +311,22 @@ constexpr int kHubBucketWide = 12;
 // query whatever the number of queries, until they fill the GPU; one warp
 // per query takes time in proportion to it. On a 300k-site torus (queries
 // half in the box, half near the surface; us for one lane / one warp per
-// query at 30,000 and 60,000 queries, the locality sort included):
-//   k = 1: 98 / 93, 99 / 147     k = 8: 185 / 146, 189 / 247
-//   k = 16: 274 / 208, 291 / 357   k = 32: 501 / 312, 532 / 547
-// and on a 200k-site patch cloud with trees, at 60,000 and 200,000 queries:
-//   k = 1: 250 / 174, 341 / 479   k = 8: 438 / 291, 639 / 828
-//   k = 16: 643 / 429, 989 / 1282   k = 32: 1024 / 687, 1901 / 2090
+// query at 40,000 and 80,000 queries, the locality sort included):
+//   k = 1: 102 / 102, 103 / 163     k = 8: 184 / 159, 198 / 277
+//   k = 16: 273 / 214, 297 / 379    k = 32: 503 / 323, 555 / 576
+// and on a 200k-site patch cloud with trees, at 100,000 and 150,000:
+//   k = 1: 278 / 256, 311 / 359     k = 8: 492 / 418, 527 / 599
+//   k = 16: 706 / 629, 789 / 909    k = 32: 1145 / 1012, 1547 / 1471
 // A lane that scans a list of hundreds of entries takes as long as one that
-// gives up at a tree (12k-site patch cloud, longest list 757, no trees: k = 4
-// 340 / 157, 371 / 430), so such clouds take the second line too.
+// gives up at a tree (12k-site patch cloud, longest list 757, no trees, 60,000
+// queries at k = 4: 340 / 157), so such clouds take that line too.
 // Register groups of 4, 8 and 16 lanes are slower than both at every size
 // (100,000 queries, k = 16: 1,638 / 994 / 837 us against 320), so the rule
 // never takes them.
 constexpr int kHubBucketLong = 9;  // a list of 2^9 - 1 entries or more
 int64_t one_lane_min_queries(int k, int hub, bool trees) {
-  const int64_t q = 32768 + 896 * (int64_t)k;
-  return (trees || hub >= kHubBucketLong) ? q * 5 / 2 : q;
+  const int64_t q = 40960 + 1100 * (int64_t)k;
+  return (trees || hub >= kHubBucketLong) ? q + 81920 : q;
 }
 
 }  // namespace

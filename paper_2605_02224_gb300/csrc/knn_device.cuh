@@ -1062,150 +1062,150 @@ __host__ __device__ __forceinline__ int list_slots(int k) { return k <= 8 ? 8 : 
 
 // ---------------------------------------------------------------------------
 // One warp per query with the candidate list N in shared memory (for large
-// k, where one list per thread would leave a few warps per SM). The list is
-// the warp's KC keys (KC = 32, 64 or 128 >= k), ascending, pads past cnt;
-// lane l owns positions l + 32 j. A row is read 32 entries at a time
-// (one coalesced 512-byte load of inlined entries); in the descent the
-// first strictly closer entry in list order is the lowest lane that votes
-// closer. In the expansion each lane whose entry falls below the k-th key
-// searches the list for it (a binary search in shared memory, all such
-// lanes at once): most of them are already in N (at k = 100, 781 of 948
-// per query on the 1M torus), and only the new ones are inserted, one at a
-// time by the whole warp: every lane compares its J keys, the votes give
-// the position, and the tail moves up by one slot. Expanded flags are kept
-// by position, the same in every lane.
+// k, where one list per thread would leave a few warps per SM, and for
+// launches with few queries). The list is the warp's KC keys (KC = 32, 64 or
+// 128 >= k), ascending, pads in the unused positions; lane l owns positions
+// l + 32 j. A key is the distance's bits above twice the rank; its lowest
+// bit, set once the entry's list has been expanded, moves with it and does
+// not change its place in the order. Pads have it set.
+__device__ __forceinline__ uint64_t warp_key(float d, int s) {
+  return pack_key(d, (uint32_t)s << 1);
+}
+
 template <int KC>
 struct WarpList {
   static constexpr int J = KC / 32;
   uint64_t* L;          // the warp's KC keys in shared memory
-  int cnt;
-  uint32_t done[J];     // bit b of word j: position 32 j + b expanded
-  uint64_t worst;       // key of position k-1 (a pad while cnt < k)
+  int from;             // every entry before this position has been expanded
+  uint64_t worst;       // key of position k-1 (a pad while fewer than k entries)
 
   __device__ __forceinline__ void init(uint64_t* list, int lane) {
     L = list;
-    cnt = 0;
+    from = 0;
 #pragma unroll
-    for (int j = 0; j < J; ++j) {
-      done[j] = 0;
-      L[lane + 32 * j] = kPadKey;
-    }
+    for (int j = 0; j < J; ++j) L[lane + 32 * j] = kPadKey;
     worst = kPadKey;
     __syncwarp();
   }
-  // bits at position pos and above move up by one (an insertion at pos)
-  __device__ __forceinline__ void open_flag(int pos) {
-    const int wi = pos >> 5, bi = pos & 31;
-#pragma unroll
-    for (int j = J - 1; j >= 0; --j) {
-      if (j > wi) {
-        done[j] = (done[j] << 1) | (j > 0 ? (done[j > 0 ? j - 1 : 0] >> 31) : 0u);
-      } else if (j == wi) {
-        const uint32_t f = done[j];
-        const uint32_t low = bi ? (f & (~0u >> (32 - bi))) : 0u;
-        done[j] = low | ((f >> bi) << 1 << bi);
+  __device__ __forceinline__ uint32_t low(int p) const { return ((const uint32_t*)L)[2 * p]; }
+  __device__ __forceinline__ uint32_t high(int p) const { return ((const uint32_t*)L)[2 * p + 1]; }
+  // Marks the nearest entry among the first k-1 not yet expanded and, with
+  // TWO, the next one, and returns how many there were; their sites in a and
+  // b (the same in every lane).
+  template <bool TWO>
+  __device__ __forceinline__ int next(int k, int lane, int& a, int& b) {
+    for (int p0 = from & ~31; p0 < k - 1; p0 += 32) {
+      const uint32_t lo = low(p0 + lane);
+      uint32_t open = __ballot_sync(0xffffffffu, p0 + lane < k - 1 && !(lo & 1u));
+      if (open == 0u) continue;
+      int w = __ffs((int)open) - 1, found = 1;
+      a = (int)(__shfl_sync(0xffffffffu, lo, w) >> 1);
+      open &= open - 1u;
+      bool mark = lane == w;
+      if (TWO && open) {
+        w = __ffs((int)open) - 1;
+        b = (int)(__shfl_sync(0xffffffffu, lo, w) >> 1);
+        mark = mark || lane == w;
+        found = 2;
       }
+      if (mark) ((uint32_t*)L)[2 * (p0 + lane)] = lo | 1u;
+      from = p0 + w + 1;
+      __syncwarp();
+      return found;
     }
+    from = k - 1;
+    return 0;
   }
-  __device__ __forceinline__ void set_flag(int pos) {
-#pragma unroll
-    for (int j = 0; j < J; ++j)
-      if (j == (pos >> 5)) done[j] |= 1u << (pos & 31);
-  }
-  // first position below lim not yet expanded, or -1
-  __device__ __forceinline__ int first_clear(int lim) const {
-    int r = -1;
-#pragma unroll
-    for (int j = J - 1; j >= 0; --j) {
-      const int nb = max(0, min(32, lim - 32 * j));
-      const uint32_t c = ~done[j] & (nb == 32 ? ~0u : ((1u << nb) - 1u));
-      if (c) r = 32 * j + __ffs((int)c) - 1;
-    }
-    return r;
-  }
-  // is key c in the list? pos: the number of keys below c (called by any
-  // subset of lanes)
+  // is key c (c < worst) in the list? pos: the number of keys below c
+  // (called by any subset of lanes). The halving steps compare distances
+  // alone: one word and one comparison each.
   __device__ __forceinline__ bool contains(uint64_t c, int& pos) const {
+    const uint32_t ch = (uint32_t)(c >> 32), cl = (uint32_t)c;
     pos = 0;
 #pragma unroll
     for (int step = KC / 2; step >= 1; step >>= 1)
-      if (L[pos + step - 1] < c) pos += step;
-    return L[pos] == c;
-  }
-  // Inserts key c, not in the list and below the k-th key, at position pos
-  // (the number of keys below it; the same in every lane; called by the
-  // whole warp).
-  __device__ __forceinline__ void insert_at(uint64_t c, int pos, int k, int lane) {
-    uint64_t prev[J];
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-      const int p = lane + 32 * j;
-      prev[j] = (p > pos && p < k) ? L[p - 1] : 0ull;
+      if (high(pos + step - 1) < ch) pos += step;
+    uint32_t l = low(pos);
+    if (high(pos) != ch) return false;
+    while (l < cl) {  // equal distances in rank order; ends at the k-th key at the latest
+      l = low(++pos);
+      if (high(pos) != ch) return false;
     }
-    __syncwarp();  // every lane has read its previous keys
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-      const int p = lane + 32 * j;
-      if (p < k) {
-        if (p > pos)
-          L[p] = prev[j];
-        else if (p == pos)
-          L[p] = c;
-      }
-    }
-    __syncwarp();
-    open_flag(pos);
-    if (cnt < k) cnt++;
-    if (cnt == k) worst = L[k - 1];
+    return (l | 1u) == (cl | 1u);
   }
-  // Offers the lanes' keys with `fresh` set (below the k-th key, not in the
-  // list; positions from contains) one after another, lowest lane first:
-  // each one still below the k-th key goes in at its position, and the
-  // positions of the keys after it that are larger move up by one.
-  __device__ __forceinline__ void offer(bool fresh, uint64_t key, int pos, int k, int lane) {
+  // Merges the lanes' keys with `fresh` set (not in the list; positions from
+  // contains) into the list in one pass: each key goes to its position plus
+  // the number of fresh keys below it, each entry moves up by the number of
+  // fresh keys below it, and what reaches position k drops out. Equal fresh
+  // keys go in once. Called by the whole warp.
+  __device__ __forceinline__ void merge(bool fresh, uint64_t key, int pos, int k, int lane) {
     uint32_t b = __ballot_sync(0xffffffffu, fresh);
-    while (b) {
-      const int j = __ffs((int)b) - 1;
-      b &= b - 1;
-      const uint64_t c = __shfl_sync(0xffffffffu, key, j);
-      const int at = __shfl_sync(0xffffffffu, pos, j);
-      if (c < worst) {
-        insert_at(c, at, k, lane);
-        if (key > c) ++pos;
-      }
-    }
-  }
-  // Inserts key c (the same in every lane; called by the whole warp) unless
-  // present; keeps k entries.
-  __device__ __forceinline__ void insert(uint64_t c, int k, int lane) {
-    uint64_t old[J], prev[J];
-    int less = 0;
-    bool eq = false;
+    if (b == 0u) return;
+    int up[J], below = 0, lowest = KC;
 #pragma unroll
-    for (int j = 0; j < J; ++j) {
-      const int p = lane + 32 * j;
-      old[j] = L[p];
-      prev[j] = p ? L[p - 1] : 0ull;
-      less += __popc(__ballot_sync(0xffffffffu, old[j] < c));
-      eq |= old[j] == c;
-    }
-    if (__any_sync(0xffffffffu, eq) || less >= k) return;
-    const int pos = less;
-    __syncwarp();  // every lane has read its old and previous keys
+    for (int j = 0; j < J; ++j) up[j] = 0;
+    do {
+      const int f = __ffs((int)b) - 1;
+      const uint64_t kf = __shfl_sync(0xffffffffu, key, f);
+      const int pf = __shfl_sync(0xffffffffu, pos, f);
+      const uint32_t same = __ballot_sync(0xffffffffu, fresh && key == kf);
+      if (lane != f && ((same >> lane) & 1u)) fresh = false;
+      b &= ~same;
+      below += kf < key ? 1 : 0;
+      lowest = min(lowest, pf);
 #pragma unroll
-    for (int j = 0; j < J; ++j) {
-      const int p = lane + 32 * j;
-      if (p < k) {
-        if (p > pos)
-          L[p] = prev[j];
-        else if (p == pos)
-          L[p] = c;
+      for (int j = 0; j < J; ++j) up[j] += pf <= lane + 32 * j ? 1 : 0;
+    } while (b);
+    uint64_t v[J];
+#pragma unroll
+    for (int j = 0; j < J; ++j)
+      if (32 * j + 31 >= lowest) v[j] = L[lane + 32 * j];
+    __syncwarp();  // every lane has read its entries
+#pragma unroll
+    for (int j = 0; j < J; ++j)
+      if (32 * j + 31 >= lowest) {
+        const int p = lane + 32 * j + up[j];
+        if (up[j] && p < k) L[p] = v[j];
       }
-    }
+    if (fresh && pos + below < k) L[pos + below] = key;
     __syncwarp();
-    open_flag(pos);
-    if (cnt < k) cnt++;
-    if (cnt == k) worst = L[k - 1];
+    from = min(from, lowest);
+    worst = L[k - 1];
+  }
+  // Inserts key c (the same in every lane) unless present.
+  __device__ __forceinline__ void insert(uint64_t c, int k, int lane) {
+    int pos = 0;
+    if (!(c < worst) || contains(c, pos)) return;
+    merge(lane == 0, c, pos, k, lane);
+  }
+};
+
+// The descent's sites: lane t holds the key of the t-th one. Each is closer
+// than all before it, so they become the list in reverse, with no search and
+// no shift; when they do not come in that order (float32 near-ties) or are
+// more than 32, they go to the list and the rest is inserted there.
+template <int KC>
+struct DescentKeys {
+  uint64_t mine, last;
+  int n;  // keys held, or -1 once they are in the list
+
+  __device__ __forceinline__ void add(uint64_t c, WarpList<KC>& N, int k, int lane) {
+    if (n >= 0 && (n == 32 || (n > 0 && c >= last))) flush(N, k, lane);
+    if (n < 0) {
+      N.insert(c, k, lane);
+      return;
+    }
+    if (lane == n) mine = c;
+    last = c;
+    ++n;
+  }
+  __device__ __forceinline__ void flush(WarpList<KC>& N, int k, int lane) {
+    if (n < 0) return;
+    const uint64_t c = __shfl_sync(0xffffffffu, mine, (n - 1 - lane) & 31);
+    if (lane < min(n, k)) N.L[lane] = c;
+    __syncwarp();
+    N.worst = N.L[k - 1];
+    n = -1;
   }
 };
 
@@ -1359,10 +1359,10 @@ __device__ __forceinline__ void hub_offer(const CloudDev& C, int hub, float qx, 
         const float4 ps = __ldg(C.hub_ent + D.x + 32 * chunk + lane);
         const int s = __float_as_int(ps.w);
         const float d = sqd32(qx, qy, qz, ps);
-        const uint64_t key = pack_key(d, (uint32_t)s);
+        const uint64_t key = warp_key(d, s);
         int pos = 0;
         const bool fresh = s < m && key < N.worst && !N.contains(key, pos);
-        N.offer(fresh, key, pos, k, lane);
+        N.merge(fresh, key, pos, k, lane);
       });
 }
 
@@ -1372,8 +1372,30 @@ constexpr int kHubStackWords = 34 * kHubMaxLevels;
 // 64-bit words of shared memory for one warp of knn_query_warp<KC>.
 __host__ __device__ constexpr int kWarpListWords(int kc) { return kc + kHubStackWords / 2; }
 
-// One query by one warp (every lane calls it with the same query). With
-// TREES (a cloud whose hub_of is not NULL) a list with a box tree is
+// Resident 256-thread blocks per SM that the one-warp kernels are held to
+// (100,000 mixed queries on a 300k-site torus, us with 3 / 4 / 5 blocks: k =
+// 100 2967 / 2446 / 2524, k = 64 - / 1532 / 1348, k = 16 - / 550 / 477).
+constexpr int kWarpBlocks(int kc, bool trees) { return (kc == 128 || trees) ? 4 : 5; }
+
+// One query by one warp (every lane calls it with the same query). The
+// descent reads its list 32 entries at a time; the first strictly closer
+// entry in list order is the lowest lane that votes closer. The expansion
+// reads the lists of the two nearest sites not yet expanded at once, 16
+// lanes each (any order of expansion is exact, and the lists average 15
+// entries), or one list with 32 lanes when only one is left; each lane whose
+// entry falls below the k-th key searches N for it, all at once (most are
+// already in N: at k = 100, 781 of 948 per query on the 1M torus), and the
+// new ones are merged in one pass.
+//
+// The kernel is bound by instruction issue. With one list at a time, each new
+// key inserted by itself (the tail moved and four flag words shifted every
+// time) and every site of the descent searched for its place, a query took
+// 40k warp instructions at k = 100; 100,000 surface queries on the 1M torus
+// took 4.01 ms, 2.36 now; 10,007 queries at k = 8 79 us with the sort, 70 now;
+// 64 queries 19 us, 16 now (there the chain of dependent loads binds: the next
+// list's bounds are asked for before the site is put into the list).
+//
+// With TREES (a cloud whose hub_of is not NULL) a list with a box tree is
 // searched through the tree (after kHubScanFirst entries in the descent);
 // the result is the same as the scan's. The walk's code costs registers
 // and issue slots in the scan loop too, so clouds without trees run the
@@ -1385,84 +1407,91 @@ __device__ __forceinline__ void knn_query_warp(const CloudDev& C, float qx, floa
                                                int32_t* __restrict__ out_idx,
                                                float* __restrict__ out_d2, int32_t row) {
   const int lane = (int)(threadIdx.x & 31u);
+  const float4 kNone = make_float4(0.f, 0.f, 0.f, __int_as_float(0x7fffffff));
   WarpList<KC> N;
   N.init(list, lane);
-  float dcur = sqd32(qx, qy, qz, __ldg(C.pts));
-  N.insert(pack_key(dcur, 0u), k, lane);
-  int cur = 0;  // the descent's current site, -1 once it is over
-  int2 rr = __ldg(C.rows);
-  int hub = -1;  // the current list's tree, or -1
-  if constexpr (TREES) hub = __ldg(C.hub_of);
-  int base = rr.x, end = rr.y;
-  for (;;) {
-    bool via_tree = false;
-    if constexpr (TREES) via_tree = hub >= 0 && (cur < 0 || base - rr.x >= kHubScanFirst);
-    if (via_tree) {
-      if constexpr (TREES) {  // the list through its tree
-        if (cur >= 0) {
-          float bd;
-          const int b = hub_first_closer(C, hub, qx, qy, qz, dcur, cur, m, lane,
-                                         (uint32_t*)(list + KC), bd);
-          if (b >= 0) {
-            cur = b;
-            dcur = bd;
-            const uint64_t kb = pack_key(bd, (uint32_t)b);
-            if (kb < N.worst) N.insert(kb, k, lane);
-            rr = __ldg(C.rows + cur);
-            base = rr.x;
-            end = rr.y;
-            hub = __ldg(C.hub_of + cur);
-            continue;
-          }
-          cur = -1;
-        } else {
-          hub_offer(C, hub, qx, qy, qz, m, k, N, lane, (uint32_t*)(list + KC));
-        }
-      }
-    } else {
-      const int e = base + lane;
-      const bool valid = e < end;
-      float4 ps = make_float4(0.f, 0.f, 0.f, __int_as_float(0x7fffffff));
-      if (valid) ps = __ldg(C.ent + e);
-      const int s = __float_as_int(ps.w);
-      const bool inr = valid && s < m;  // rows ascend: past the first s >= m nothing is
-      const float d = sqd32(qx, qy, qz, ps);
-      const uint64_t key = pack_key(d, (uint32_t)s);
-      const bool row_done = __any_sync(0xffffffffu, valid && !inr) || base + 32 >= end;
-      if (cur >= 0) {
-        const bool cl = inr && strictly_closer_at(C, qx, qy, qz, d, s, dcur, cur);
+
+  // ---- Algorithm 1
+  {
+    DescentKeys<KC> T;
+    T.n = 0;
+    T.mine = T.last = kPadKey;
+    int2 rr = __ldg(C.rows);
+    int hub = -1;  // the current list's tree, or -1
+    if constexpr (TREES) hub = __ldg(C.hub_of);
+    float dcur = sqd32(qx, qy, qz, __ldg(C.pts));
+    int cur = 0;
+    T.add(warp_key(dcur, 0), N, k, lane);
+    int base = rr.x;
+    for (;;) {
+      int to = -1;  // the site moved to
+      float dto = 0.f;
+      bool over = base >= rr.y;
+      if (TREES && hub >= 0 && base - rr.x >= kHubScanFirst) {
+        to = hub_first_closer(C, hub, qx, qy, qz, dcur, cur, m, lane, (uint32_t*)(list + KC), dto);
+        over = true;
+      } else if (!over) {
+        const int e = base + lane;
+        const float4 ps = e < rr.y ? __ldg(C.ent + e) : kNone;
+        const int s = __float_as_int(ps.w);
+        const float d = sqd32(qx, qy, qz, ps);
+        // rows ascend: past the first s >= m nothing is below m
+        const bool cl = s < m && strictly_closer_at(C, qx, qy, qz, d, s, dcur, cur);
         const uint32_t b = __ballot_sync(0xffffffffu, cl);
+        over = base + 32 >= rr.y || __any_sync(0xffffffffu, s >= m);
         if (b) {
           const int w = __ffs((int)b) - 1;
-          cur = __shfl_sync(0xffffffffu, s, w);
-          dcur = __shfl_sync(0xffffffffu, d, w);
-          const uint64_t kw = __shfl_sync(0xffffffffu, key, w);
-          if (kw < N.worst) N.insert(kw, k, lane);
-          rr = __ldg(C.rows + cur);
-          base = rr.x;
-          end = rr.y;
-          if constexpr (TREES) hub = __ldg(C.hub_of + cur);
-          continue;
+          to = __shfl_sync(0xffffffffu, s, w);
+          dto = __shfl_sync(0xffffffffu, d, w);
         }
-        if (row_done) cur = -1;
-      } else {
-        int pos = 0;
-        const bool fresh = inr && key < N.worst && !N.contains(key, pos);
-        N.offer(fresh, key, pos, k, lane);
-      }
-      if (!row_done) {
         base += 32;
+      }
+      if (to >= 0) {
+        rr = __ldg(C.rows + to);
+        if constexpr (TREES) hub = __ldg(C.hub_of + to);
+        cur = to;
+        dcur = dto;
+        T.add(warp_key(dto, to), N, k, lane);
+        base = rr.x;
+      } else if (over) {
+        break;
+      }
+    }
+    T.flush(N, k, lane);
+  }
+
+  // ---- Algorithm 2
+  for (;;) {
+    int site = 0, other = 0;
+    // clouds with trees: one list at a time (the second may have a tree)
+    const int lists = N.template next<!TREES>(k, lane, site, other);
+    if (lists == 0) break;
+    if constexpr (TREES) {
+      const int hub = __ldg(C.hub_of + site);
+      if (hub >= 0) {
+        hub_offer(C, hub, qx, qy, qz, m, k, N, lane, (uint32_t*)(list + KC));
         continue;
       }
     }
-    const int pos = N.first_clear(min(N.cnt, k - 1));
-    if (pos < 0) break;
-    N.set_flag(pos);
-    const int site = (int)(uint32_t)N.L[pos];
-    rr = __ldg(C.rows + site);
-    base = rr.x;
-    end = rr.y;
-    if constexpr (TREES) hub = __ldg(C.hub_of + site);
+    const int width = lists == 2 ? 16 : 32;
+    if (lists == 2 && lane >= 16) site = other;
+    const int2 rr = __ldg(C.rows + site);
+    const uint32_t group = width == 32 ? 0xffffffffu : (lane < 16 ? 0xffffu : 0xffff0000u);
+    int e = rr.x + (lane & (width - 1));
+    int end = rr.y;
+    for (;;) {
+      const float4 ps = e < end ? __ldg(C.ent + e) : kNone;
+      const int s = __float_as_int(ps.w);
+      const float d = sqd32(qx, qy, qz, ps);
+      const uint64_t key = warp_key(d, s);
+      int pos = 0;
+      const bool fresh = s < m && key < N.worst && !N.contains(key, pos);
+      const uint32_t stop = __ballot_sync(0xffffffffu, s >= m);
+      N.merge(fresh, key, pos, k, lane);
+      e += width;
+      if (stop & group) end = 0;  // the list's end, or its first entry out of the prefix
+      if (!__any_sync(0xffffffffu, e < end)) break;
+    }
   }
   int32_t* oi = out_idx + (int64_t)row * k;
   float* od = out_d2 + (int64_t)row * k;
@@ -1470,9 +1499,9 @@ __device__ __forceinline__ void knn_query_warp(const CloudDev& C, float qx, floa
   for (int j = 0; j < KC / 32; ++j) {
     const int p = lane + 32 * j;
     if (p < k) {
-      const bool real = p < N.cnt;
       const uint64_t key = N.L[p];
-      __stcs(oi + p, real ? (int32_t)(uint32_t)key : -1);
+      const bool real = key != kPadKey;
+      __stcs(oi + p, real ? (int32_t)((uint32_t)key >> 1) : -1);
       __stcs(od + p, real ? __uint_as_float((uint32_t)(key >> 32)) : __int_as_float(0x7f800000));
     }
   }

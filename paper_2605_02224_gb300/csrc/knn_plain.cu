@@ -236,7 +236,7 @@ cudaError_t run_smem(const CloudDevHost& c, const PlainLaunch& L, cudaStream_t s
 // warp: 8 KB per 256-thread block at KC = 128). One block per 8 queries of
 // the processing order, started by the hardware wherever a block ends.
 template <int KC, bool TREES>
-__global__ void __launch_bounds__(kThreads) knn_plain_warp_kernel(
+__global__ void __launch_bounds__(kThreads, kWarpBlocks(KC, TREES)) knn_plain_warp_kernel(
     CloudDev C, const float* __restrict__ q, int q_stride, int64_t nq, int k,
     const int32_t* __restrict__ mq, int m_scalar, const int32_t* __restrict__ perm,
     int32_t* __restrict__ out_idx, float* __restrict__ out_d2, int32_t* __restrict__ err,

@@ -71,8 +71,8 @@ def test_default_lanes_around_the_crossover(surface, n, k):
     order = W.permutation(n, 82)
     c = Cloud.build(P, order).upload()
     lo, hi = W.padded_box(P)
-    base = 32768 + 896 * k
-    for nq in (base - 1, base, base * 5 // 2 - 1, base * 5 // 2):
+    base = 40960 + 1100 * k
+    for nq in (base - 1, base, base + 81919, base + 81920):
         q = torch.from_numpy(W.box_queries(nq, 83, lo, hi)).cuda()
         want = c.knn(q, k, lanes=32, placement=1)
         runs = [c.knn(q, k), c.knn(q, k, lanes=1, placement=2)]
@@ -86,3 +86,34 @@ def test_default_lanes_around_the_crossover(surface, n, k):
         for i, d in runs:
             assert torch.equal(i, want[0]) and torch.equal(d, want[1])
     c.close()
+
+
+@pytest.mark.parametrize("k", [1, 2, 3, 17, 31, 32, 33, 64, 65, 128])
+def test_one_warp_lists(k):
+    """Two lists read at once and merged in one pass, on clouds where they
+    share entries and keys tie: a lattice (whole rings at one distance),
+    duplicated points, patches with box trees, and clouds of fewer sites than
+    k; queries on sites, at cell centres and in the box, bounds from 1 up.
+    The rows are the register kernel's, and the oracle's."""
+    import torch
+    L, _ = W.lattice(9)
+    S, _ = W.sphere(300, 91)
+    P, _ = W.patches4(30000, 92)
+    for pts in (L, np.concatenate([S, S, S[:100]]), P, S[:5], S[:40]):
+        n = len(pts)
+        order = W.permutation(n, 93)
+        c = Cloud.build(pts, order).upload()
+        lo, hi = W.padded_box(pts)
+        Q = np.concatenate([W.box_queries(150, 94, lo, hi), pts[:: max(1, n // 150)][:150],
+                            (pts[:50] + np.float32(0.5))]).astype(np.float32)
+        m = np.random.default_rng(95).integers(1, n + 1, len(Q)).astype(np.int32)
+        m[::3] = n
+        q, mt = torch.from_numpy(Q).cuda(), torch.from_numpy(m).cuda()
+        lanes = 32 if k <= 64 else 16
+        want = c.knn(q, k, mt, lanes=lanes, placement=1)
+        got = c.knn(q, k, mt, lanes=32, placement=2)
+        torch.cuda.synchronize()
+        assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1]), (n, k)
+        parity.check_rows(pts[order], Q, k, m, got[0].cpu().numpy(), got[1].cpu().numpy(),
+                          rows=range(0, len(Q), 11))
+        c.close()
