@@ -1089,32 +1089,21 @@ struct WarpList {
   }
   __device__ __forceinline__ uint32_t low(int p) const { return ((const uint32_t*)L)[2 * p]; }
   __device__ __forceinline__ uint32_t high(int p) const { return ((const uint32_t*)L)[2 * p + 1]; }
-  // Marks the nearest entry among the first k-1 not yet expanded and, with
-  // TWO, the next one, and returns how many there were; their sites in a and
-  // b (the same in every lane).
-  template <bool TWO>
-  __device__ __forceinline__ int next(int k, int lane, int& a, int& b) {
+  // Marks the nearest entry among the first k-1 not yet expanded and returns
+  // its site, or -1 (the same in every lane).
+  __device__ __forceinline__ int next(int k, int lane) {
     for (int p0 = from & ~31; p0 < k - 1; p0 += 32) {
       const uint32_t lo = low(p0 + lane);
-      uint32_t open = __ballot_sync(0xffffffffu, p0 + lane < k - 1 && !(lo & 1u));
+      const uint32_t open = __ballot_sync(0xffffffffu, p0 + lane < k - 1 && !(lo & 1u));
       if (open == 0u) continue;
-      int w = __ffs((int)open) - 1, found = 1;
-      a = (int)(__shfl_sync(0xffffffffu, lo, w) >> 1);
-      open &= open - 1u;
-      bool mark = lane == w;
-      if (TWO && open) {
-        w = __ffs((int)open) - 1;
-        b = (int)(__shfl_sync(0xffffffffu, lo, w) >> 1);
-        mark = mark || lane == w;
-        found = 2;
-      }
-      if (mark) ((uint32_t*)L)[2 * (p0 + lane)] = lo | 1u;
+      const int w = __ffs((int)open) - 1;
+      if (lane == w) ((uint32_t*)L)[2 * (p0 + lane)] = lo | 1u;
       from = p0 + w + 1;
       __syncwarp();
-      return found;
+      return (int)(__shfl_sync(0xffffffffu, lo, w) >> 1);
     }
     from = k - 1;
-    return 0;
+    return -1;
   }
   // is key c (c < worst) in the list? pos: the number of keys below c
   // (called by any subset of lanes). The halving steps compare distances
@@ -1136,8 +1125,8 @@ struct WarpList {
   // Merges the lanes' keys with `fresh` set (not in the list; positions from
   // contains) into the list in one pass: each key goes to its position plus
   // the number of fresh keys below it, each entry moves up by the number of
-  // fresh keys below it, and what reaches position k drops out. Equal fresh
-  // keys go in once. Called by the whole warp.
+  // fresh keys below it, and what reaches position k drops out. Called by the
+  // whole warp, with no two fresh keys equal.
   __device__ __forceinline__ void merge(bool fresh, uint64_t key, int pos, int k, int lane) {
     uint32_t b = __ballot_sync(0xffffffffu, fresh);
     if (b == 0u) return;
@@ -1148,9 +1137,7 @@ struct WarpList {
       const int f = __ffs((int)b) - 1;
       const uint64_t kf = __shfl_sync(0xffffffffu, key, f);
       const int pf = __shfl_sync(0xffffffffu, pos, f);
-      const uint32_t same = __ballot_sync(0xffffffffu, fresh && key == kf);
-      if (lane != f && ((same >> lane) & 1u)) fresh = false;
-      b &= ~same;
+      b &= b - 1u;
       below += kf < key ? 1 : 0;
       lowest = min(lowest, pf);
 #pragma unroll
@@ -1372,28 +1359,32 @@ constexpr int kHubStackWords = 34 * kHubMaxLevels;
 // 64-bit words of shared memory for one warp of knn_query_warp<KC>.
 __host__ __device__ constexpr int kWarpListWords(int kc) { return kc + kHubStackWords / 2; }
 
-// Resident 256-thread blocks per SM that the one-warp kernels are held to
-// (100,000 mixed queries on a 300k-site torus, us with 3 / 4 / 5 blocks: k =
-// 100 2967 / 2446 / 2524, k = 64 - / 1532 / 1348, k = 16 - / 550 / 477).
+// Resident 256-thread blocks per SM that the one-warp kernels are held to.
+// Five (48 registers) hide more latency in large launches, four (64) run the
+// single query faster; us with 4 / 5 blocks: 100,000 queries at k = 100 2530 /
+// 2402, 64 queries 105 / 125; on a 300k-site torus 100,000 queries at k = 64
+// 1532 / 1348, at k = 16 550 / 477, 64 queries the same; with trees, k = 32,
+// 10,000 queries 276 / 292, 60,000 609 / 546.
 constexpr int kWarpBlocks(int kc, bool trees) { return (kc == 128 || trees) ? 4 : 5; }
 
 // One query by one warp (every lane calls it with the same query). The
 // descent reads its list 32 entries at a time; the first strictly closer
-// entry in list order is the lowest lane that votes closer. The expansion
-// reads the lists of the two nearest sites not yet expanded at once, 16
-// lanes each (any order of expansion is exact, and the lists average 15
-// entries), or one list with 32 lanes when only one is left; each lane whose
-// entry falls below the k-th key searches N for it, all at once (most are
-// already in N: at k = 100, 781 of 948 per query on the 1M torus), and the
-// new ones are merged in one pass.
+// entry in list order is the lowest lane that votes closer. In the expansion
+// each lane whose entry falls below the k-th key searches N for it, all at
+// once (most are already in N: at k = 100, 781 of 948 per query on the 1M
+// torus), and the new ones are merged in one pass.
 //
-// The kernel is bound by instruction issue. With one list at a time, each new
-// key inserted by itself (the tail moved and four flag words shifted every
-// time) and every site of the descent searched for its place, a query took
-// 40k warp instructions at k = 100; 100,000 surface queries on the 1M torus
-// took 4.01 ms, 2.36 now; 10,007 queries at k = 8 79 us with the sort, 70 now;
-// 64 queries 19 us, 16 now (there the chain of dependent loads binds: the next
-// list's bounds are asked for before the site is put into the list).
+// The kernel is bound by instruction issue. With each new key inserted by
+// itself (the tail moved and four flag words shifted every time) and every
+// site of the descent searched for its place, a query took 40k warp
+// instructions at k = 100; 100,000 surface queries on the 1M torus took 4.01
+// ms, 2.56 now; 10,007 queries at k = 8 79 us with the sort, 68 now; 64
+// queries 19 us, 17 now (there the chain of dependent loads binds: the next
+// list's bounds are asked for before the site is put into the list). Reading
+// the lists of two sites at once, 16 lanes each, took 2.36 ms at k = 100 and
+// was slower up to k = 16; it can expand a site that would have dropped out
+// by its turn, which changes rows whose distances all tie within float32
+// rounding, so lists are read one at a time.
 //
 // With TREES (a cloud whose hub_of is not NULL) a list with a box tree is
 // searched through the tree (after kHubScanFirst entries in the descent);
@@ -1462,10 +1453,8 @@ __device__ __forceinline__ void knn_query_warp(const CloudDev& C, float qx, floa
 
   // ---- Algorithm 2
   for (;;) {
-    int site = 0, other = 0;
-    // clouds with trees: one list at a time (the second may have a tree)
-    const int lists = N.template next<!TREES>(k, lane, site, other);
-    if (lists == 0) break;
+    const int site = N.next(k, lane);
+    if (site < 0) break;
     if constexpr (TREES) {
       const int hub = __ldg(C.hub_of + site);
       if (hub >= 0) {
@@ -1473,24 +1462,18 @@ __device__ __forceinline__ void knn_query_warp(const CloudDev& C, float qx, floa
         continue;
       }
     }
-    const int width = lists == 2 ? 16 : 32;
-    if (lists == 2 && lane >= 16) site = other;
     const int2 rr = __ldg(C.rows + site);
-    const uint32_t group = width == 32 ? 0xffffffffu : (lane < 16 ? 0xffffu : 0xffff0000u);
-    int e = rr.x + (lane & (width - 1));
-    int end = rr.y;
-    for (;;) {
-      const float4 ps = e < end ? __ldg(C.ent + e) : kNone;
+    for (int e = rr.x + lane, base = rr.x; base < rr.y; base += 32, e += 32) {
+      const float4 ps = e < rr.y ? __ldg(C.ent + e) : kNone;
       const int s = __float_as_int(ps.w);
       const float d = sqd32(qx, qy, qz, ps);
       const uint64_t key = warp_key(d, s);
       int pos = 0;
       const bool fresh = s < m && key < N.worst && !N.contains(key, pos);
-      const uint32_t stop = __ballot_sync(0xffffffffu, s >= m);
+      // the list's end, or its first entry out of the prefix
+      const bool over = __any_sync(0xffffffffu, s >= m);
       N.merge(fresh, key, pos, k, lane);
-      e += width;
-      if (stop & group) end = 0;  // the list's end, or its first entry out of the prefix
-      if (!__any_sync(0xffffffffu, e < end)) break;
+      if (over) break;
     }
   }
   int32_t* oi = out_idx + (int64_t)row * k;

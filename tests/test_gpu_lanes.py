@@ -90,8 +90,8 @@ def test_default_lanes_around_the_crossover(surface, n, k):
 
 @pytest.mark.parametrize("k", [1, 2, 3, 17, 31, 32, 33, 64, 65, 128])
 def test_one_warp_lists(k):
-    """Two lists read at once and merged in one pass, on clouds where they
-    share entries and keys tie: a lattice (whole rings at one distance),
+    """New keys merged in one pass, on clouds where lists share entries and
+    keys tie: a lattice (whole rings at one distance),
     duplicated points, patches with box trees, and clouds of fewer sites than
     k; queries on sites, at cell centres and in the box, bounds from 1 up.
     The rows are the register kernel's, and the oracle's."""
