@@ -237,8 +237,9 @@ typedef struct {
   int32_t lanes;        /* lanes per query: 0 = default (32 from k = 48
                            up, in batches below about 41,000 + 1,100 k
                            queries - 82,000 more on clouds with long
-                           successor lists - and on clouds with very long
-                           lists and no box trees; else 1), or
+                           successor lists, 33,000 more for each k above
+                           32 - and on clouds with very long lists and
+                           no box trees; else 1), or
                            1, 4, 8, 16, 32 (4 and 8 hold k <= 64; one
                            lane above 64 needs placement 2 and no
                            counters) */

@@ -88,16 +88,34 @@ __device__ __forceinline__ uint64_t* smem_column(int kcap) {
   return batch_lists + (size_t)warp * kcap * 32 + lane;
 }
 
+// The warp's next work unit of a segment: `item` moves on to the unit's item
+// (a warp's units only grow), begin and end are its queries. False when the
+// segment is done. Called by the whole warp.
+__device__ __forceinline__ bool next_unit(const Item* __restrict__ items, int nitems,
+                                          uint32_t units, unsigned* next, int& item, int& begin,
+                                          int& end) {
+  unsigned u = 0;
+  if ((threadIdx.x & 31u) == 0) u = atomicAdd(next, 1u);
+  u = __shfl_sync(0xffffffffu, u, 0);
+  if (u >= units) return false;
+  while (item + 1 < nitems && u >= __ldg(&items[item + 1].first)) ++item;
+  const int per = __ldg(&items[item].per);
+  begin = (int)((u - __ldg(&items[item].first)) * (unsigned)per);
+  end = begin + min(per, __ldg(&items[item].nq) - begin);
+  return true;
+}
+
 // DEFER: a query that meets a list with a box tree is handed over
 // (appended to the plan's list of its class) instead of answered.
 template <class L, bool DEFER>
-__device__ __forceinline__ void serve_item_smem(const ReqDev& R, const Item& w, uint64_t* col) {
+__device__ __forceinline__ void serve_item_smem(const ReqDev& R, int req, int begin, int end,
+                                                uint64_t* col) {
   const int lane = (int)(threadIdx.x & 31u);
   const CloudDev C{R.pts, R.rows, R.succ, R.n, R.ent, DEFER ? R.hub_of : nullptr};
   const int k = R.k;
-  for (int i0 = w.begin; i0 < w.end; i0 += 32) {
+  for (int i0 = begin; i0 < end; i0 += 32) {
     const int i = i0 + lane;
-    bool live = i < w.end;
+    bool live = i < end;
     int64_t qi = 0;
     float qx = 0.f, qy = 0.f, qz = 0.f;
     int m = 0;
@@ -125,7 +143,7 @@ __device__ __forceinline__ void serve_item_smem(const ReqDev& R, const Item& w, 
     if constexpr (DEFER) {
       if (gave_up) {
         const int c = handover_class(k);
-        R.ho->list[c][atomicAdd(&R.ho->count[c], 1)] = make_int2(w.req, (int)qi);
+        R.ho->list[c][atomicAdd(&R.ho->count[c], 1)] = make_int2(req, (int)qi);
       }
     }
     __syncwarp();
@@ -133,12 +151,12 @@ __device__ __forceinline__ void serve_item_smem(const ReqDev& R, const Item& w, 
 }
 
 template <int G, int S>
-__device__ __forceinline__ void serve_item(const ReqDev& R, const Item& w) {
+__device__ __forceinline__ void serve_item(const ReqDev& R, int begin, int end) {
   const Grp<G> g;
   const int gi = (int)((threadIdx.x & 31u) / G);
   constexpr int kGroups = 32 / G;
   const CloudDev C{R.pts, R.rows, R.succ, R.n, R.ent};
-  for (int i = w.begin + gi; i < w.end; i += kGroups) {
+  for (int i = begin + gi; i < end; i += kGroups) {
     const int64_t qi = R.perm ? (int64_t)__ldg(R.perm + i) : (int64_t)i;
     const float* qp = R.q + qi * R.q_stride;
     const float qx = __ldg(qp), qy = __ldg(qp + 1), qz = __ldg(qp + 2);
@@ -161,18 +179,13 @@ __device__ __forceinline__ void serve_item(const ReqDev& R, const Item& w) {
 template <int G, int S>
 __global__ void __launch_bounds__(kThreads, S <= 2 ? 5 : (S <= 4 ? 4 : 3)) knn_batch_group_kernel(const ReqDev* __restrict__ reqs,
                                                                    const Item* __restrict__ items,
-                                                                   int nitems,
-                                                                   int* __restrict__ next,
+                                                                   int nitems, uint32_t units,
+                                                                   unsigned* __restrict__ next,
                                                                    int kcap) {
   (void)kcap;  // lists in registers
-  const uint32_t lane = threadIdx.x & 31u;
-  for (;;) {
-    int it = 0;
-    if (lane == 0) it = atomicAdd(next, 1);
-    it = __shfl_sync(0xffffffffu, it, 0);
-    if (it >= nitems) return;
-    const Item w = items[it];
-    serve_item<G, S>(reqs[w.req], w);
+  int item = 0, begin, end;
+  while (next_unit(items, nitems, units, next, item, begin, end)) {
+    serve_item<G, S>(reqs[items[item].req], begin, end);
     __syncwarp();
   }
 }
@@ -184,25 +197,22 @@ __global__ void __launch_bounds__(kThreads, S <= 2 ? 5 : (S <= 4 ? 4 : 3)) knn_b
 template <int THREADS, int W, int LK, bool DEFER>
 __global__ void __launch_bounds__(THREADS, THREADS == 256 ? (LK == 0 ? 3 : 5) : 1) knn_batch_smem_kernel(const ReqDev* __restrict__ reqs,
                                                                  const Item* __restrict__ items,
-                                                                 int nitems,
-                                                                 int* __restrict__ next,
+                                                                 int nitems, uint32_t units,
+                                                                 unsigned* __restrict__ next,
                                                                  int kcap) {
-  const uint32_t lane = threadIdx.x & 31u;
   uint64_t* col = smem_column(kcap);
-  for (;;) {
-    int it = 0;
-    if (lane == 0) it = atomicAdd(next, 1);
-    it = __shfl_sync(0xffffffffu, it, 0);
-    if (it >= nitems) return;
-    const Item w = items[it];
+  int item = 0, begin, end;
+  while (next_unit(items, nitems, units, next, item, begin, end)) {
+    const int req = __ldg(&items[item].req);
+    const ReqDev& R = reqs[req];
     if constexpr (LK == 8)
-      serve_item_smem<PermList<8>, DEFER>(reqs[w.req], w, col);
+      serve_item_smem<PermList<8>, DEFER>(R, req, begin, end, col);
     else if constexpr (LK == 16)
-      serve_item_smem<PermList<16>, DEFER>(reqs[w.req], w, col);
+      serve_item_smem<PermList<16>, DEFER>(R, req, begin, end, col);
     else if constexpr (W == 1)
-      serve_item_smem<PermList32, DEFER>(reqs[w.req], w, col);
+      serve_item_smem<PermList32, DEFER>(R, req, begin, end, col);
     else
-      serve_item_smem<SortedList<32 * W, W>, DEFER>(reqs[w.req], w, col);
+      serve_item_smem<SortedList<32 * W, W>, DEFER>(R, req, begin, end, col);
   }
 }
 
@@ -212,23 +222,19 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? (LK == 0 ? 3 : 5) : 
 template <int KC, bool TREES>
 __global__ void __launch_bounds__(kThreads, kWarpBlocks(KC, TREES)) knn_batch_warp_kernel(const ReqDev* __restrict__ reqs,
                                                                   const Item* __restrict__ items,
-                                                                  int nitems,
-                                                                  int* __restrict__ next,
+                                                                  int nitems, uint32_t units,
+                                                                  unsigned* __restrict__ next,
                                                                   int kcap) {
   (void)kcap;
   __shared__ uint64_t lists[kThreads / 32][TREES ? kWarpListWords(KC) : KC];
   const int warp = (int)(threadIdx.x >> 5);
   const uint32_t lane = threadIdx.x & 31u;
-  for (;;) {
-    int it = 0;
-    if (lane == 0) it = atomicAdd(next, 1);
-    it = __shfl_sync(0xffffffffu, it, 0);
-    if (it >= nitems) return;
-    const Item w = items[it];
-    const ReqDev& R = reqs[w.req];
+  int item = 0, begin, end;
+  while (next_unit(items, nitems, units, next, item, begin, end)) {
+    const ReqDev& R = reqs[__ldg(&items[item].req)];
     const CloudDev C{R.pts,    R.rows,     R.succ,    R.n,       R.ent,
                      R.hub_of, R.hub_desc, R.hub_ent, R.hub_node};
-    for (int i = w.begin; i < w.end; ++i) {
+    for (int i = begin; i < end; ++i) {
       const int64_t qi = R.perm ? (int64_t)__ldg(R.perm + i) : (int64_t)i;
       const float* qp = R.q + qi * R.q_stride;
       const float qx = __ldg(qp), qy = __ldg(qp + 1), qz = __ldg(qp + 2);
@@ -314,6 +320,8 @@ constexpr int kHubBucketWide = 12;
 // query at 40,000 and 80,000 queries, the locality sort included):
 //   k = 1: 102 / 102, 103 / 163     k = 8: 184 / 159, 198 / 277
 //   k = 16: 273 / 214, 297 / 379    k = 32: 503 / 323, 555 / 576
+// above k = 32, where the one-lane list moves keys, at 100,000 and 400,000:
+//   k = 40: 1204 / 874, 2949 / 3249   k = 47: 1473 / 987, 4116 / 3689
 // and on a 200k-site patch cloud with trees, at 100,000 and 150,000:
 //   k = 1: 278 / 256, 311 / 359     k = 8: 492 / 418, 527 / 599
 //   k = 16: 706 / 629, 789 / 909    k = 32: 1145 / 1012, 1547 / 1471
@@ -325,7 +333,8 @@ constexpr int kHubBucketWide = 12;
 // never takes them.
 constexpr int kHubBucketLong = 9;  // a list of 2^9 - 1 entries or more
 int64_t one_lane_min_queries(int k, int hub, bool trees) {
-  const int64_t q = 40960 + 1100 * (int64_t)k;
+  int64_t q = 40960 + 1100 * (int64_t)k;
+  if (k > 32) q += 32768 * (int64_t)(k - 32);
   return (trees || hub >= kHubBucketLong) ? q + 81920 : q;
 }
 
@@ -418,7 +427,7 @@ const void* variant_kernel(int variant, int kcap) {
 
 }  // namespace
 
-BatchLaunch batch_config(int nitems, int blocks_per_sm, int kcap, int variant) {
+BatchLaunch batch_config(int64_t units, int blocks_per_sm, int kcap, int variant) {
   ensure_smem_attributes();  // an error shows again at launch
   BatchLaunch b;
   b.variant = variant;
@@ -435,20 +444,22 @@ BatchLaunch batch_config(int nitems, int blocks_per_sm, int kcap, int variant) {
   }
   const int per_sm = blocks_per_sm > 0 ? std::min(blocks_per_sm, occ) : occ;
   const int wpb = b.threads / 32;
-  const int64_t blocks_needed = ((int64_t)std::max(1, nitems) + wpb - 1) / wpb;
+  const int64_t blocks_needed = (std::max<int64_t>(1, units) + wpb - 1) / wpb;
   b.grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms() * per_sm, blocks_needed));
   return b;
 }
 
-cudaError_t launch_batch_kernel(const ReqDev* d_reqs, const Item* d_items, int nitems, int* d_next,
-                                const BatchLaunch& b, cudaStream_t s) {
-  if (nitems <= 0) return cudaSuccess;
+cudaError_t launch_batch_kernel(const ReqDev* d_reqs, const Item* d_items, int nitems,
+                                uint32_t units, unsigned* d_next, const BatchLaunch& b,
+                                cudaStream_t s) {
+  if (units == 0) return cudaSuccess;
   const cudaError_t ae = ensure_smem_attributes();
   if (ae != cudaSuccess) return ae;
   const void* fn = variant_kernel(b.variant, b.kcap);
   if (!fn) return cudaErrorInvalidValue;
   int kcap = b.kcap;
-  void* args[] = {(void*)&d_reqs, (void*)&d_items, (void*)&nitems, (void*)&d_next, (void*)&kcap};
+  void* args[] = {(void*)&d_reqs, (void*)&d_items, (void*)&nitems,
+                  (void*)&units,  (void*)&d_next,  (void*)&kcap};
   return cudaLaunchKernel(fn, dim3((unsigned)b.grid), dim3((unsigned)b.threads), args, b.smem, s);
 }
 
@@ -479,7 +490,14 @@ std::vector<Segment> make_segments(std::vector<Item>& items, int blocks_per_sm,
     Segment g;
     g.begin = i;
     g.count = j - i;
-    g.launch = batch_config(g.count, blocks_per_sm, kcap, items[i].variant);
+    int64_t units = 0;
+    for (int t = i; t < j; ++t) {
+      items[t].first = (uint32_t)units;
+      units += ((int64_t)items[t].nq + items[t].per - 1) / items[t].per;
+      if (units > kMaxUnits) return {};
+    }
+    g.units = (uint32_t)units;
+    g.launch = batch_config(units, blocks_per_sm, kcap, items[i].variant);
     segs.push_back(g);
     i = j;
   }
@@ -528,7 +546,7 @@ void SideStreams::destroy() {
   *this = SideStreams{};
 }
 
-cudaError_t launch_segments(const ReqDev* d_reqs, const Item* d_items, int* d_next,
+cudaError_t launch_segments(const ReqDev* d_reqs, const Item* d_items, unsigned* d_next,
                             const std::vector<Segment>& segs, cudaStream_t s,
                             const SideStreams& side, int64_t queries) {
   const bool split = segs.size() > 1 && side.fork && queries <= kSplitMaxQueries;
@@ -540,7 +558,7 @@ cudaError_t launch_segments(const ReqDev* d_reqs, const Item* d_items, int* d_ne
   for (size_t i = 0; i < segs.size() && e == cudaSuccess; ++i) {
     const Segment& g = segs[i];
     const int on = (int)(i % (size_t)(nside + 1));
-    e = launch_batch_kernel(d_reqs, d_items + g.begin, g.count, d_next + i, g.launch,
+    e = launch_batch_kernel(d_reqs, d_items + g.begin, g.count, g.units, d_next + i, g.launch,
                             on ? side.s[on - 1] : s);
   }
   for (int i = 0; i < nside && e == cudaSuccess; ++i) {
@@ -577,7 +595,7 @@ struct mknn_batch {
   Item* d_items = nullptr;
   int64_t nitems = 0;
   std::vector<Segment> segs;
-  int* d_next = nullptr;         // [i] queue of segment i
+  unsigned* d_next = nullptr;    // [i] queue of segment i
   void* d_ws = nullptr;          // sort scratch: shared histogram, per-request cells and orders
   size_t ws_bytes = 0;
   std::vector<size_t> cell_off, perm_off;  // per request, 0 if not sorted
@@ -730,12 +748,14 @@ mknn_status mknn_batch_create(const mknn_batch_req* reqs, int32_t nreq,
       ho_cap[handover_class(reqs[r].k)] += reqs[r].nq;
       b->ho_class[handover_class(reqs[r].k)] = true;
     }
-    const int per = item_queries(b->lanes[r], rounds);
-    for (int64_t s0 = 0; s0 < reqs[r].nq; s0 += per)
-      items.push_back(Item{r, (int32_t)s0, (int32_t)std::min<int64_t>(reqs[r].nq, s0 + per), v});
+    if (reqs[r].nq > 0)
+      items.push_back(Item{r, v, 0u, (int32_t)reqs[r].nq,
+                           item_queries(b->lanes[r], rounds, reqs[r].nq)});
   }
   b->segs = make_segments(items, o.blocks_per_sm, req_k);
-  b->nitems = (int64_t)items.size();
+  if (b->segs.empty() && !items.empty())
+    return bfail(MKNN_ENOMEM, "more work items than one launch can count");
+  for (const Segment& g : b->segs) b->nitems += (int64_t)g.units;
   cudaError_t e;
   if ((e = cudaMalloc((void**)&b->d_reqs, sizeof(ReqDev) * std::max(nreq, 1))) != cudaSuccess ||
       (e = cudaMalloc((void**)&b->d_items, sizeof(Item) * std::max<size_t>(items.size(), 1))) !=

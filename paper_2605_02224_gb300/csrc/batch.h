@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <vector>
 
@@ -50,18 +51,29 @@ cudaError_t launch_handover(const ReqDev* d_reqs, Handover* d_ho, int c, int gri
 // stride within an item (at most 256 queries) then stays below 2^31 - 1.
 constexpr int64_t kRequestQueryLimit = (int64_t)0x7FFFFFFF - 256;
 
-// A contiguous range of one request's queries (in processing order),
-// served by one warp with kernel variant `variant`.
+// One request's share of a segment: its queries in processing order, cut into
+// work units of `per` (the last one shorter), the unit `first` of the segment
+// first. A warp takes the next unit of its segment with one atomic and finds
+// the request it belongs to, so that neither host nor device memory holds
+// anything per unit (a 16-byte record per unit, built, sorted and copied for
+// each pack, took the server 6.8 of 9.5 ms for 64 requests).
 struct Item {
-  int32_t req, begin, end, variant;
+  int32_t req, variant;
+  uint32_t first;
+  int32_t nq, per;
 };
+// The segment's number of units stays below this: its counter goes past it
+// by one per warp.
+constexpr int64_t kMaxUnits = (int64_t)0xFFFFFFFF - (1 << 20);
 
 // Variant index for lanes-per-query G, capacity k and list placement
 // (2 = shared memory, 1 = registers; only 32 lanes have both), or -1.
 int variant_index(int lanes, int k, int placement);
-// Queries per work item for the given lanes and rounds per item.
-inline int item_queries(int lanes, int rounds) { return (32 / lanes) * rounds; }
-// Rounds per work item (a warp answers its item's queries one round after
+// Queries per work unit for the given lanes and rounds per unit, at most nq.
+inline int item_queries(int lanes, int rounds, int64_t nq) {
+  return (int)std::min<int64_t>((int64_t)(32 / lanes) * rounds, nq);
+}
+// Rounds per work unit (a warp answers its unit's queries one round after
 // another): one. Longer items hold up the end of a persistent launch and,
 // with groups of lanes on clouds with hub rows, let one slow query hold up
 // the rest of its item. On the 64-cloud batching workload (57.6M queries)
@@ -115,22 +127,26 @@ struct BatchLaunch {
   int kcap = 0;       // list capacity: the largest k among the launch's requests
   int variant = kSmemVariant;
 };
-// Grid, block and shared memory for `nitems` items of one variant.
-BatchLaunch batch_config(int nitems, int blocks_per_sm, int kcap, int variant);
-// Launches the persistent kernel of b.variant; *d_next must be zero on entry.
-cudaError_t launch_batch_kernel(const ReqDev* d_reqs, const Item* d_items, int nitems, int* d_next,
-                                const BatchLaunch& b, cudaStream_t s);
+// Grid, block and shared memory for `units` work units of one variant.
+BatchLaunch batch_config(int64_t units, int blocks_per_sm, int kcap, int variant);
+// Launches the persistent kernel of b.variant over `units` work units of
+// `nitems` items; *d_next must be zero on entry.
+cudaError_t launch_batch_kernel(const ReqDev* d_reqs, const Item* d_items, int nitems,
+                                uint32_t units, unsigned* d_next, const BatchLaunch& b,
+                                cudaStream_t s);
 
 // The items of one variant: a contiguous range of the item array with its
 // own queue counter and launch.
 struct Segment {
   int begin = 0, count = 0;
+  uint32_t units = 0;
   BatchLaunch launch;
 };
 // Reorders items by variant (the one-lane kernels' first, larger lists
-// before smaller; each class's items in their given order) and returns one segment per variant present;
-// req_k[r] is request r's k (a one-lane segment's list capacity is its
-// largest k).
+// before smaller; each class's items in their given order), numbers their
+// units and returns one segment per variant and list class present, or none
+// when one would have more than kMaxUnits units; req_k[r] is request r's k (a
+// one-lane segment's list capacity is its largest k).
 std::vector<Segment> make_segments(std::vector<Item>& items, int blocks_per_sm,
                                    const std::vector<int>& req_k);
 // Streams beside a launch's own for its segments, and the events that fork
@@ -152,7 +168,7 @@ struct SideStreams {
 // streams, the plan of 12 clouds (0.76M queries, three one-lane segments)
 // 4.22 ms in turn and 3.30 side by side, the larger lists first.
 constexpr int64_t kSplitMaxQueries = int64_t(1) << 21;
-cudaError_t launch_segments(const ReqDev* d_reqs, const Item* d_items, int* d_next,
+cudaError_t launch_segments(const ReqDev* d_reqs, const Item* d_items, unsigned* d_next,
                             const std::vector<Segment>& segs, cudaStream_t s,
                             const SideStreams& side, int64_t queries);
 

@@ -128,11 +128,8 @@ size_t request_bytes(int64_t nq, int k) {
          sizeof(ReqDev);
 }
 
-// Room for the work items of a pack: at most one item per query and one
-// partial item per request (items may be as small as one query).
-size_t items_bytes(int64_t nq_total, size_t nreq) {
-  return al(sizeof(Item) * ((size_t)nq_total + 2 * nreq + 64));
-}
+// Room for the work items of a pack, one per request.
+size_t items_bytes(size_t nreq) { return al(sizeof(Item) * nreq); }
 
 // Room for a pack's hand-over: the lists' header and a (request, query)
 // pair per query (one-lane items on clouds with box trees).
@@ -254,7 +251,7 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
     if (e == cudaSuccess) e = cudaMemcpyAsync(dd, dbase + R.d2_off, nk, cudaMemcpyDeviceToHost, s);
   } else {
     // pack layout: [counter][histogram][ReqDev x n][Item x m][hand-over][per request data]
-    int* d_next = (int*)dbase;
+    unsigned* d_next = (unsigned*)dbase;
     void* d_hist = dbase + 256;
     const size_t reqs_off = 256 + kSortHistBytes;
     const int nreq = (int)tickets.size();
@@ -271,7 +268,7 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
       lanes[i] = o.lanes ? o.lanes : chosen.lanes;
       placement[i] = o.lanes ? default_placement(q.k, lanes[i]) : chosen.placement;
     }
-    const size_t ho_off = reqs_off + al(sizeof(ReqDev) * nreq) + items_bytes(pack_nq, nreq);
+    const size_t ho_off = reqs_off + al(sizeof(ReqDev) * nreq) + items_bytes(nreq);
     Handover* d_ho = (Handover*)(dbase + ho_off);
     int2* d_pairs = (int2*)(dbase + ho_off + al(sizeof(Handover)));
     int64_t ho_cap[3] = {0, 0, 0};
@@ -301,12 +298,11 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
         ho_cap[handover_class(q.k)] += q.nq;
         rd[i].ho = d_ho;
       }
-      const int per = item_queries(lanes[i], kItemRounds);
       req_k[i] = q.k;
-      for (int64_t b0 = 0; b0 < q.nq; b0 += per)
-        items.push_back(Item{i, (int32_t)b0, (int32_t)std::min<int64_t>(q.nq, b0 + per), v});
+      items.push_back(Item{i, v, 0u, (int32_t)q.nq, item_queries(lanes[i], kItemRounds, q.nq)});
     }
     const std::vector<Segment> segs = make_segments(items, 0, req_k);
+    if (segs.empty() && e == cudaSuccess) e = cudaErrorInvalidValue;  // too many units to count
     const size_t ni = items.size();
     const size_t items_off = reqs_off + al(sizeof(ReqDev) * nreq);
     // request table and items go through the pinned mirror
@@ -389,7 +385,7 @@ void mknn_server::run() {
       const ReqRec& R = recs[t - 1];
       const size_t rb = request_bytes(R.r.nq, R.r.k);
       const size_t meta = o.plain ? 0 : al(sizeof(ReqDev) * (take.size() + 1)) +
-                                            items_bytes(nq_total + R.r.nq, take.size() + 1) +
+                                            items_bytes(take.size() + 1) +
                                             handover_bytes(nq_total + R.r.nq);
       if (!take.empty() && (bytes + rb + meta > room || nq_total + R.r.nq > o.max_batch_queries))
         break;
@@ -402,7 +398,7 @@ void mknn_server::run() {
     if (take.empty()) continue;
     const size_t meta = o.plain ? kSortHistBytes + 256
                                 : al(sizeof(ReqDev) * take.size()) +
-                                      items_bytes(nq_total, take.size()) + handover_bytes(nq_total);
+                                      items_bytes(take.size()) + handover_bytes(nq_total);
     bytes += meta;
     size_t off = 0;
     if (!arena.alloc(bytes, &off)) continue;
@@ -420,7 +416,7 @@ void mknn_server::run() {
       R.d2_off = c;
     } else {
       size_t c = 256 + kSortHistBytes + al(sizeof(ReqDev) * take.size()) +
-                 items_bytes(nq_total, take.size()) + handover_bytes(nq_total);
+                 items_bytes(take.size()) + handover_bytes(nq_total);
       for (uint64_t t : take) {
         ReqRec& R = recs[t - 1];
         const int64_t nq = R.r.nq;
@@ -515,7 +511,10 @@ mknn_status mknn_server_submit(mknn_server* s, const mknn_request* r, uint64_t* 
   if (r->nq < 1 || r->nq >= kRequestQueryLimit || r->k < 1 || r->k > MKNN_MAX_K ||
       r->m < 0 || r->m > c->n || !r->q || !r->out_idx || !r->out_d2)
     return sfail(MKNN_EINVAL, "bad request (nq, k, m or NULL buffer)");
-  const size_t need = request_bytes(r->nq, r->k) + al(kPackFixed) + 4096 + items_bytes(r->nq, 1);
+  // with 16 bytes per query for the pack's own tables (the hand-over's pairs
+  // take 8 of them)
+  const size_t need = request_bytes(r->nq, r->k) + al(kPackFixed) + 4096 +
+                      al(16 * ((size_t)r->nq + 66));
   if (need > s->arena_bytes)
     return sfail(MKNN_ENOMEM, "request alone exceeds the server's memory budget");
   lk.unlock();
