@@ -609,7 +609,8 @@ mknn_status mknn_knn_ex(const mknn_cloud* c, const float* q, int64_t nq, int32_t
   }
   if (sort_need > 0) {
     int32_t* p = (int32_t*)((char*)ws + sort_workspace_bytes(nq));
-    cudaError_t e = launch_query_sort(c->dev(), q, q_stride, nq, ws, p, s);
+    cudaError_t e = launch_query_sort_any(c->dev(), q, q_stride, nq, ws,
+                                          (int32_t*)((char*)ws + kSortHistBytes), p, s);
     if (e != cudaSuccess) return cuda_fail(e, "query sort launch");
     perm = p;
   }

@@ -89,6 +89,15 @@ cudaError_t launch_query_sort_split(const CloudDevHost& c, const float* q, int32
                                     int64_t nq, void* hist, int32_t* cell, int32_t* perm,
                                     cudaStream_t stream);
 
+// The sort of a launch's own queries: one block for at most kSortSmallMax of
+// them, the five kernels above for more. Whole calls on a 300k-site torus at
+// k = 8, us with the five kernels / one block: 4,096 queries 53 / 35, 8,000
+// 67 / 53, 16,384 85 / 80; from about twice that one block is the slower.
+constexpr int64_t kSortSmallMax = int64_t(1) << 14;
+cudaError_t launch_query_sort_any(const CloudDevHost& c, const float* q, int32_t q_stride,
+                                  int64_t nq, void* hist, int32_t* cell, int32_t* perm,
+                                  cudaStream_t stream);
+
 // From this k up, one warp per query (its list in shared memory) is the
 // default instead of one thread per query.
 constexpr int kWarpMinK = 48;

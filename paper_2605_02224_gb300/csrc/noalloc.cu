@@ -133,7 +133,9 @@ extern "C" mknn_status mknn_knn_noalloc(const mknn_cloud* c, const float* q, int
   if (nq >= kSortMinQueries) {
     const size_t sort_bytes = sort_workspace_bytes(nq);
     perm = (int32_t*)((char*)base + align256(sort_bytes));
-    if ((e = launch_query_sort(cd, q, q_stride, nq, base, perm, s)) != cudaSuccess) {
+    if ((e = launch_query_sort_any(cd, q, q_stride, nq, base,
+                                   (int32_t*)((char*)base + kSortHistBytes), perm, s)) !=
+        cudaSuccess) {
       set_error(std::string("query sort launch: ") + cudaGetErrorString(e));
       return MKNN_ECUDA;
     }

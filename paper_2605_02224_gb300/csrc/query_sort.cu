@@ -150,9 +150,119 @@ __global__ void qsort_scatter(const int32_t* __restrict__ cell, int64_t nq,
   }
 }
 
+// The whole sort of at most kSortSmallMax queries in one block: box, cells of
+// a 32 x 32 x 16 grid, counts, their scan and the scatter, with the counts
+// (two 16-bit ones per word) in shared memory and each query's cell and its
+// place in the cell in a register. What bounds the five kernels and three
+// clears at such sizes is their launches and the gaps between them.
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallPer = (int)(kSortSmallMax / kSmallThreads);
+constexpr int kSmallCells = 1 << 14;
+__global__ void __launch_bounds__(kSmallThreads) qsort_small(const float* __restrict__ q,
+                                                             int stride, int nq,
+                                                             int32_t* __restrict__ perm) {
+  __shared__ uint32_t count[kSmallCells / 2];
+  __shared__ float part[32][6];
+  __shared__ int32_t warp_sums[32];
+  const int t = (int)threadIdx.x, lane = t & 31, warp = t >> 5;
+  float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+  for (int i = t; i < nq; i += kSmallThreads)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const float v = __ldg(q + (int64_t)i * stride + d);
+      if (v == v) {
+        lo[d] = fminf(lo[d], v);
+        hi[d] = fmaxf(hi[d], v);
+      }
+    }
+  for (int i = t; i < kSmallCells / 2; i += kSmallThreads) count[i] = 0u;
+#pragma unroll
+  for (int d = 0; d < 3; ++d)
+    for (int o = 16; o > 0; o >>= 1) {
+      lo[d] = fminf(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
+      hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
+    }
+  if (lane == 0)
+    for (int d = 0; d < 3; ++d) {
+      part[warp][d] = lo[d];
+      part[warp][3 + d] = hi[d];
+    }
+  __syncthreads();
+  float sc[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    lo[d] = part[lane][d];
+    hi[d] = part[lane][3 + d];
+    for (int o = 16; o > 0; o >>= 1) {
+      lo[d] = fminf(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
+      hi[d] = fmaxf(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
+    }
+    const float ext = hi[d] - lo[d];
+    sc[d] = ext > 0.f ? (d < 2 ? 32.f : 16.f) / ext : 0.f;
+  }
+  uint32_t at[kSmallPer];  // cell, and the query's place in it from bit 14 up
+#pragma unroll
+  for (int j = 0; j < kSmallPer; ++j) {
+    const int i = t + j * kSmallThreads;
+    at[j] = 0u;
+    if (i < nq) {
+      const float* p = q + (int64_t)i * stride;
+      // a NaN coordinate maps to 0 (fminf/fmaxf drop NaN operands)
+      const float fx = fminf(fmaxf((__ldg(p) - lo[0]) * sc[0], 0.f), 31.f);
+      const float fy = fminf(fmaxf((__ldg(p + 1) - lo[1]) * sc[1], 0.f), 31.f);
+      const float fz = fminf(fmaxf((__ldg(p + 2) - lo[2]) * sc[2], 0.f), 15.f);
+      // Morton order: 4 bits of z below the highest bits of x and y
+      const uint32_t x = (uint32_t)fx, y = (uint32_t)fy;
+      const uint32_t c = spread3(x & 15u) | (spread3(y & 15u) << 1) |
+                         (spread3((uint32_t)fz) << 2) | ((x >> 4) << 12) | ((y >> 4) << 13);
+      const int sh = 16 * (int)(c & 1u);
+      const uint32_t old = atomicAdd(&count[c >> 1], 1u << sh);
+      at[j] = c | (((old >> sh) & 0xffffu) << 14);
+    }
+  }
+  __syncthreads();
+  // exclusive scan of the counts: 16 cells per thread
+  constexpr int kWords = kSmallCells / 2 / kSmallThreads;
+  uint32_t w[kWords];
+  int32_t sum = 0, total = 0;
+#pragma unroll
+  for (int j = 0; j < kWords; ++j) {
+    w[j] = count[t * kWords + j];
+    sum += (int32_t)((w[j] & 0xffffu) + (w[j] >> 16));
+  }
+  uint32_t run = (uint32_t)block_exclusive_scan(sum, warp_sums, &total);
+#pragma unroll
+  for (int j = 0; j < kWords; ++j) {  // offsets are below nq <= 2^14
+    const uint32_t a = run, b = a + (w[j] & 0xffffu);
+    count[t * kWords + j] = a | (b << 16);
+    run = b + (w[j] >> 16);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kSmallPer; ++j) {
+    const int i = t + j * kSmallThreads;
+    if (i < nq) {
+      const uint32_t c = at[j] & (uint32_t)(kSmallCells - 1);
+      const uint32_t off = (count[c >> 1] >> (16 * (int)(c & 1u))) & 0xffffu;
+      perm[off + (at[j] >> 14)] = i;
+    }
+  }
+}
+static_assert(kSortSmallMax == kSmallCells, "16-bit counts and offsets hold kSortSmallMax");
+
 inline size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 }  // namespace
+
+cudaError_t launch_query_sort_any(const CloudDevHost& c, const float* q, int32_t q_stride,
+                                  int64_t nq, void* hist, int32_t* cell, int32_t* perm,
+                                  cudaStream_t stream) {
+  if (nq == 0) return cudaSuccess;
+  if (nq > kSortSmallMax)
+    return launch_query_sort_split(c, q, q_stride, nq, hist, cell, perm, stream);
+  qsort_small<<<1, kSmallThreads, 0, stream>>>(q, q_stride, (int)nq, perm);
+  return cudaGetLastError();
+}
 
 size_t sort_workspace_bytes(int64_t nq) { return kSortHistBytes + align256((size_t)nq * 4); }
 

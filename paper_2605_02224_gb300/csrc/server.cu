@@ -328,9 +328,9 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
     for (int i = 0; i < nreq && e == cudaSuccess; ++i) {
       const ReqRec& R = recs[tickets[i] - 1];
       if (R.r.nq >= kSortMinQueries)
-        e = launch_query_sort_split(clouds[R.r.cloud]->dev(), (const float*)(dbase + R.q_off), 3,
-                                    R.r.nq, d_hist, (int32_t*)(dbase + R.cell_off),
-                                    (int32_t*)(dbase + R.perm_off), s);
+        e = launch_query_sort_any(clouds[R.r.cloud]->dev(), (const float*)(dbase + R.q_off), 3,
+                                  R.r.nq, d_hist, (int32_t*)(dbase + R.cell_off),
+                                  (int32_t*)(dbase + R.perm_off), s);
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(d_next, 0, segs.size() * sizeof(int), s);
     // the segments on the slot's stream and its side streams, joined before

@@ -117,3 +117,32 @@ def test_one_warp_lists(k):
         parity.check_rows(pts[order], Q, k, m, got[0].cpu().numpy(), got[1].cpu().numpy(),
                           rows=range(0, len(Q), 11))
         c.close()
+
+
+@pytest.mark.parametrize("nq", [1, 33, 1023, 4096, 16383, 16384, 16385])
+@pytest.mark.parametrize("shape", ["box", "one", "line", "odd"])
+def test_sorted_rows_equal_unsorted(cloud, nq, shape):
+    """The one-block sort and the five-kernel one around the line between
+    them: every query's row is written, and is the unsorted launch's, for
+    queries in a box, all at one point, on a line, and with coordinates that
+    are not finite."""
+    import torch
+    c, _ = cloud
+    Q = W.box_queries(nq, 74, [-1.6] * 3, [1.6] * 3)
+    if shape == "one":
+        Q[:] = Q[0]
+    elif shape == "line":
+        Q[:, 1:] = Q[0, 1:]
+    elif shape == "odd":
+        Q[::3, 0] = np.nan
+        Q[1::5, 1] = np.inf
+        Q[2::7, 2] = -np.inf
+    q = torch.from_numpy(Q).cuda()
+    q4 = torch.cat([q, q[:, :1]], 1).contiguous()
+    want = c.knn(q, 4, sort=-1)
+    idx, d2 = torch.full_like(want[0], -9), torch.full_like(want[1], -9)
+    M.mknn_knn_noalloc(c.handle, q, nq, 3, 4, None, 0, idx, d2)
+    for got in (c.knn(q4, 4, sort=1), (idx, d2)):
+        torch.cuda.synchronize()
+        assert torch.equal(got[0], want[0])
+        assert torch.equal(got[1].view(torch.int32), want[1].view(torch.int32))
