@@ -157,6 +157,10 @@ struct SideStreams {
   cudaEvent_t fork = nullptr, join[kSideStreams] = {};
   bool create();   // false when the driver refuses; destroy() is still due
   void destroy();
+  // The first n side streams continue after what is queued on `from`; and
+  // `from` after what is queued on them.
+  cudaError_t fork_from(cudaStream_t from, int n) const;
+  cudaError_t join_to(cudaStream_t from, int n) const;
 };
 // Launches every segment, segment i draining the queue counter d_next[i]
 // (zero on entry). The segments of a launch of at most kSplitMaxQueries
