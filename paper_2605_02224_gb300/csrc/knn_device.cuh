@@ -634,6 +634,7 @@ __device__ __forceinline__ uint64_t lane_key(float d, int s) { return pack_key(d
 // list's capacity cap); positions in [cap, KS) read as pads without a load.
 template <int KS, int W>
 struct SortedList {
+  static constexpr int kVoteEvery = 1;  // see knn_query_smem
   uint64_t* col;
   int cap;
   int cnt;
@@ -698,6 +699,7 @@ struct PermWord<16> {
 // insertion position: no key moves, a fixed instruction sequence.
 template <int S>
 struct PermList {
+  static constexpr int kVoteEvery = 2;  // see knn_query_smem
   using T = typename PermWord<S>::T;
   uint64_t* col;
   T perm;          // bits 4j..4j+3: the slot of position j
@@ -753,6 +755,7 @@ struct PermList {
 // bounds it is the list's 256 bytes per thread: 24 warps per SM, so the block
 // is held to three per SM and takes the registers it wants (72, no spills).
 struct PermList32 {
+  static constexpr int kVoteEvery = 1;  // see knn_query_smem
   uint64_t* col;      // slot s at col[s * 32], s >= 32 - k
   uint64_t near, far; // bits 4j..4j+3: the slot of position j (16 + j: less 16)
   uint32_t done;      // by position
@@ -888,7 +891,9 @@ __device__ __forceinline__ void load_pair(const float4* p, float4& a, float4& b)
 // other; a bounded number of scan steps keeps the waiting lanes from
 // standing by while one lane reads a list of thousands (plan of 12 clouds:
 // 4.50 ms with 8 steps, 5.97 ms unbounded; 3 / 5 / 8 / 16 steps on the
-// torus batch: 6.19 / 6.07 / 6.04 / 6.05 ms).
+// torus batch: 6.19 / 6.07 / 6.04 / 6.05 ms). Lists of up to 16 vote on it
+// every second step (6.04 to 5.97 ms; with longer lists, where fewer warps
+// are resident, 2.53 to 2.60 ms at k = 32).
 //
 // Why pairs: entries come from the inlined table (site and rank in 16
 // bytes), two in one 32-byte load at an even index, the next pair in flight
@@ -896,8 +901,13 @@ __device__ __forceinline__ void load_pair(const float4* p, float4& a, float4& b)
 // L1 lines touched (8,700 to 4,600 per warp; L1 takes about one line per
 // cycle). A pair may begin before the row (skip) or reach past its end.
 //
-// 4M queries, 1M-site torus, k = 16: 9.12 ms with the one-loop form, 6.04 ms
-// now; 1M queries, 300k-site bumpy sphere, k = 4: 0.98 to 0.58 ms.
+// 4M queries, 1M-site torus, k = 16: 9.12 ms with the one-loop form, 5.97 ms
+// now; 1M queries, 300k-site bumpy sphere, k = 4: 0.98 to 0.58 ms. What binds
+// now is latency: most pairs come from L2, and a row switch is two dependent
+// loads. Loading the next pair only after a hit is decided (four registers
+// fewer) takes 6.84 ms; asking for a moved-to row's bounds before the
+// insertion (two registers more, spills) 6.21 ms; prefetching a row's second
+// pair, or every next one, to L1 6.10 and 6.55 ms.
 //
 // DEFER (a cloud with box trees over its long lists, hub_of not NULL): a
 // query gives up, with nothing written (the function returns true), when it
@@ -955,25 +965,27 @@ __device__ __forceinline__ bool knn_query_smem(const CloudDev& C, bool live, flo
   if (open >= 0) open_row();
   while (act) {
     const int na = __popc(act);
-    for (int step = 0; step < kScanSteps; ++step) {
+    for (int step = 0; step < kScanSteps; step += L::kVoteEvery) {
       const uint32_t waiting = __ballot_sync(0xffffffffu, ev != 0u) & act;
       if (3 * __popc(waiting) >= 2 * na) break;
-      if (ev == 0u) {
-        d0 = sqd32(qx, qy, qz, a);
-        d1 = sqd32(qx, qy, qz, b);
-        s0 = __float_as_int(a.w);
-        s1 = __float_as_int(b.w);
-        const bool more = e + 2 < end && s1 < m;
-        if (!skip && s0 < m && !(d0 > thr)) ev = kHit0;
-        skip = 0;
-        if (e + 1 < end && s1 < m && !(d1 > thr)) ev |= kHit1;
-        if (more) {
-          e += 2;
-          load_pair(C.ent + e, a, b);
-        } else {
-          ev |= kRowEnd;
+#pragma unroll
+      for (int t = 0; t < L::kVoteEvery; ++t)
+        if (ev == 0u) {
+          d0 = sqd32(qx, qy, qz, a);
+          d1 = sqd32(qx, qy, qz, b);
+          s0 = __float_as_int(a.w);
+          s1 = __float_as_int(b.w);
+          const bool more = e + 2 < end && s1 < m;
+          if (!skip && s0 < m && !(d0 > thr)) ev = kHit0;
+          skip = 0;
+          if (e + 1 < end && s1 < m && !(d1 > thr)) ev |= kHit1;
+          if (more) {
+            e += 2;
+            load_pair(C.ent + e, a, b);
+          } else {
+            ev |= kRowEnd;
+          }
         }
-      }
     }
     if (ev != 0u && ev != kIdle) {
       if (ev & (kHit0 | kHit1)) {
