@@ -103,8 +103,7 @@ constexpr int kWarpVariant32 = 16;
 // kTreeVariant32 + 0, 1, 2.
 constexpr int kTreeVariant32 = 19;
 // The variant a request runs: a one-warp variant turns into its tree form
-// when the request's cloud has trees, and with `handover` (plans, not the
-// server's packs) a one-lane variant into its hand-over form. variant_index
+// when the request's cloud has trees, and with `handover` a one-lane variant into its hand-over form. variant_index
 // never returns these forms (it picks the first of equal variants).
 inline int with_trees(int v, bool trees, bool handover = false) {
   if (!trees) return v;

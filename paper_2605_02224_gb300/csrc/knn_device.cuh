@@ -835,22 +835,10 @@ __device__ __forceinline__ uint64_t list_key(const PermList<S>& N, int p, int k)
   return N.key_at(p, k);
 }
 
-// Descent decision: is the candidate at squared distance d (site ps)
-// strictly closer than the current site (dcur, pc)? float32 outside the
-// guard band, float64 in the oracle's order inside it.
-__device__ __forceinline__ bool strictly_closer(float qx, float qy, float qz, float d, float4 ps,
-                                                float dcur, float4 pc) {
-  if (dcur >= kTiny) {
-    if (d < dcur * (1.f - kGuard)) return true;
-    if (d > dcur * (1.f + kGuard)) return false;
-  } else if (d > 2.f * kTiny) {
-    return false;
-  }
-  return sqd64(qx, qy, qz, ps.x, ps.y, ps.z) < sqd64(qx, qy, qz, pc.x, pc.y, pc.z);
-}
-
-// strictly_closer with both sites given by their ranks: the coordinates are
-// loaded only when the float32 decision is inside the guard band.
+// Descent decision: is site s, at squared distance d, strictly closer than
+// the current site cur, at dcur? float32 outside the guard band; inside it the
+// coordinates are loaded and the distances compared in float64, in the
+// oracle's order.
 __device__ __forceinline__ bool strictly_closer_at(const CloudDev& C, float qx, float qy, float qz,
                                                    float d, int s, float dcur, int cur) {
   if (dcur >= kTiny) {
@@ -1303,7 +1291,7 @@ __device__ __forceinline__ void hub_walk(const CloudDev& C, int4 D, int lane, ui
 // site is strictly closer than the current one (rank cur, squared distance
 // dcur) - the first such entry of the list in rank order - or -1; its
 // squared distance goes to bd. A box is skipped when its nearest point is
-// beyond the float32 distance above which strictly_closer says no, or its
+// beyond the float32 distance above which strictly_closer_at says no, or its
 // smallest rank is not below m or below the best found.
 __device__ __forceinline__ int hub_first_closer(const CloudDev& C, int hub, float qx, float qy,
                                                 float qz, float dcur, int cur, int m, int lane,

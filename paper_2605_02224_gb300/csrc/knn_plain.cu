@@ -116,8 +116,9 @@ cudaError_t run_thread(const CloudDevHost& c, const PlainLaunch& L, cudaStream_t
 // k = 16: 6.45 ms with 4; 1M bumpy queries at k = 4: 0.62 ms with 4, 0.59 ms
 // with 6, 0.57 ms with 5). Lists of 32 slots leave room for three blocks.
 // LK: the list kind (8: PermList<8>, k <= 8; 16: PermList<16>, 9 <= k <= 16;
-// 0: PermList32, k <= 32, or SortedList searched over 32 W). DEFER (a cloud with box trees): a query that gives up (knn_query_smem) is appended
-// to defer[0 .. *ndefer) for the one-warp kernel.
+// 0: PermList32, k <= 32, or SortedList searched over 32 W). DEFER (a cloud
+// with box trees): a query that gives up (knn_query_smem) is appended to
+// defer[0 .. *ndefer) for the one-warp kernel.
 template <int THREADS, int W, int LK, bool DEFER>
 __global__ void __launch_bounds__(THREADS, THREADS == 256 ? (LK == 0 ? 3 : 5) : 1) knn_plain_smem_kernel(
     CloudDev C, const float* __restrict__ q, int q_stride, int64_t nq, int k, int kcap,
@@ -443,10 +444,6 @@ int num_sms() {
   });
 }
 
-// Measured on the 1M-site torus with 4M box queries: one query per thread
-// is fastest up to k = 16 (k = 4: 359M q/s vs 264M with 8 lanes; k = 16:
-// 124M vs 111M with 16 lanes); above that the 32-slot register list costs
-// too much occupancy and 16 lanes win (k = 32: 44M vs 26M with 1 lane).
 namespace {
 
 __global__ void fill_entries_kernel(const float4* __restrict__ pts, const int32_t* __restrict__ succ,
@@ -493,11 +490,9 @@ cudaError_t launch_fill_entries(const void* pts, const int32_t* succ, int64_t E,
   return cudaGetLastError();
 }
 
-// Measured on the 1M-site torus with 4M box queries (queries/s): one query
-// per thread with the list in shared memory against one warp per query with
-// the warp's list in shared memory: k = 32: 164M / 120M; k = 64: 51M / 54M;
-// k = 100: 21M / 26M; k = 128: 12M / 21M. Register lists over a group of
-// 32 (16) lanes: 61M (45M), 21M (7M), 8M (4M), 6M (3M).
+// One query per thread against one warp per query, 100,000 mixed queries on a
+// 300k-site torus: k = 32 593 / 737 us, k = 64 2,069 / 1,349, k = 100 5,117 /
+// 2,446. Register lists over a group of 32 (16) lanes: k = 64 4,845 (14,784).
 int default_lanes(int k) { return k >= kWarpMinK ? 32 : 1; }
 
 int plain_max_k(int lanes) { return (lanes == 4 || lanes == 8) ? 64 : 128; }
