@@ -494,7 +494,10 @@ mknn_status mknn_server_add_cloud(mknn_server* s, mknn_cloud* cloud, int32_t* id
 /* Queues a request; *ticket identifies it. EINVAL for a bad request,
  * ENOMEM if it alone exceeds the memory budget. Thread-safe. */
 mknn_status mknn_server_submit(mknn_server* s, const mknn_request* req, uint64_t* ticket);
-/* *state: 0 pending, 1 done, or minus a status code if it failed. */
+/* *state: 0 pending, 1 done, or minus a status code if it failed: minus EINVAL
+ * when k is above what the server's `lanes` hold (the rest of its launch is
+ * answered), else the launch's error, which every request of the launch ends
+ * with. A failed request's rows are not written or not to be used. */
 mknn_status mknn_server_poll(mknn_server* s, uint64_t ticket, int32_t* state);
 /* Waits (at most timeout_s seconds) until every submitted request is done;
  * ETIMEOUT if the wait runs out. */

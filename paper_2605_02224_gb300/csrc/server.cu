@@ -98,6 +98,7 @@ struct ReqRec {
   Clock::time_point t_submit, t_done;
   int32_t state = 0;  // 0 pending, 1 done, <0 failed
   bool q_pinned = false, out_pinned = false;
+  mknn_status refused = MKNN_OK;  // why the pack went without this request
   // placement inside the pack's region (device and pinned staging)
   size_t q_off = 0, cell_off = 0, perm_off = 0, idx_off = 0, d2_off = 0;
 };
@@ -110,6 +111,7 @@ struct Slot {
   // host-to-device copies, after the kernels; `done` follows the copies back
   cudaEvent_t t0 = nullptr, t_h2d = nullptr, t_kern = nullptr;
   bool busy = false;
+  mknn_status status = MKNN_OK;  // of the launch: what its requests end with
   std::vector<uint64_t> tickets;
   size_t off = 0, bytes = 0;
 };
@@ -173,12 +175,16 @@ struct mknn_server {
 void mknn_server::reap_locked() {
   for (Slot& sl : slots) {
     if (!sl.busy) continue;
-    cudaError_t e = cudaEventQuery(sl.done);
+    const cudaError_t e = cudaEventQuery(sl.done);
     if (e == cudaErrorNotReady) continue;
-    const Clock::time_point now = Clock::now();
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      if (sl.status == MKNN_OK) sl.status = MKNN_ECUDA;
+    }
     for (uint64_t t : sl.tickets) {
       ReqRec& R = recs[t - 1];
-      if (e == cudaSuccess) {
+      const mknn_status st = sl.status != MKNN_OK ? sl.status : R.refused;
+      if (st == MKNN_OK) {
         if (!R.out_pinned) {
           const size_t nk = (size_t)R.r.nq * R.r.k * 4;
           std::memcpy(R.r.out_idx, h_arena + sl.off + R.idx_off, nk);
@@ -188,15 +194,14 @@ void mknn_server::reap_locked() {
         ++completed;
         queries += R.r.nq;
       } else {
-        R.state = -(int32_t)MKNN_ECUDA;
+        R.state = -(int32_t)st;
         ++failed;
       }
       R.t_done = Clock::now();
       t_last = R.t_done;
       lat.emplace_back(t, std::chrono::duration<double, std::milli>(R.t_done - R.t_submit).count());
-      (void)now;
     }
-    if (e == cudaSuccess) {
+    if (sl.status == MKNN_OK) {
       float a = 0, b = 0, c = 0;
       if (cudaEventElapsedTime(&a, sl.t0, sl.t_h2d) == cudaSuccess &&
           cudaEventElapsedTime(&b, sl.t_h2d, sl.t_kern) == cudaSuccess &&
@@ -208,7 +213,6 @@ void mknn_server::reap_locked() {
         cudaGetLastError();
       }
     }
-    if (e != cudaSuccess) cudaGetLastError();
     arena.release(sl.off, sl.bytes);
     sl.busy = false;
     sl.tickets.clear();
@@ -217,12 +221,14 @@ void mknn_server::reap_locked() {
   cv_done.notify_all();
 }
 
-// Issues one pack on a slot (called without the lock held).
+// Issues one pack on a slot (called without the lock held). What goes wrong
+// is the slot's status, which its requests end with.
 void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, size_t bytes) {
   cudaStream_t s = sl.s;
   char* dbase = d_arena + off;
   char* hbase = h_arena + off;
   cudaError_t e = cudaEventRecord(sl.t0, s);
+  sl.status = MKNN_OK;
   if (o.plain) {
     // baseline: the request alone through the plain entry point
     ReqRec& R = recs[tickets[0] - 1];
@@ -239,11 +245,11 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
     ko.lanes = o.lanes;
     ko.workspace = dbase + R.cell_off;
     ko.workspace_bytes = al((size_t)q.nq * 4) * 2 + kSortHistBytes;
-    if (e == cudaSuccess &&
-        mknn_knn_ex(clouds[q.cloud], (const float*)(dbase + R.q_off), q.nq, 3, q.k, nullptr, q.m,
-                    (int32_t*)(dbase + R.idx_off), (float*)(dbase + R.d2_off), &ko,
-                    (mknn_stream_t)s) != MKNN_OK)
-      e = cudaErrorLaunchFailure;
+    if (e == cudaSuccess)
+      sl.status = mknn_knn_ex(clouds[q.cloud], (const float*)(dbase + R.q_off), q.nq, 3, q.k,
+                              nullptr, q.m, (int32_t*)(dbase + R.idx_off),
+                              (float*)(dbase + R.d2_off), &ko, (mknn_stream_t)s);
+    if (sl.status != MKNN_OK) e = cudaErrorLaunchFailure;  // nothing to copy back
     if (e == cudaSuccess) e = cudaEventRecord(sl.t_kern, s);
     void* di = R.out_pinned ? (void*)q.out_idx : (void*)(hbase + R.idx_off);
     void* dd = R.out_pinned ? (void*)q.out_d2 : (void*)(hbase + R.d2_off);
@@ -276,6 +282,11 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
       ReqRec& R = recs[tickets[i] - 1];
       const mknn_request& q = R.r;
       const mknn_cloud* c = clouds[q.cloud];
+      const int base = variant_index(lanes[i], q.k, placement[i]);
+      if (base < 0) {  // k above what the server's lanes hold: the others go without it
+        R.refused = MKNN_EINVAL;
+        continue;
+      }
       const CloudDevHost cd = c->dev(q.k);
       const size_t qb = (size_t)q.nq * 12;
       const void* src = q.q;
@@ -292,8 +303,7 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
                      q.m ? q.m : (int32_t)c->n, (const float4*)cd.ent, cd.hub_of,
                      (const int4*)cd.hub_desc, (const float4*)cd.hub_ent,
                      (const float4*)cd.hub_node};
-      const int v =
-          with_trees(variant_index(lanes[i], q.k, placement[i]), cd.hub_of != nullptr, true);
+      const int v = with_trees(base, cd.hub_of != nullptr, true);
       if (v == kHandoverVariant || v == kHandoverVariant128) {
         ho_cap[handover_class(q.k)] += q.nq;
         rd[i].ho = d_ho;
@@ -302,7 +312,8 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
       items.push_back(Item{i, v, 0u, (int32_t)q.nq, item_queries(lanes[i], kItemRounds, q.nq)});
     }
     const std::vector<Segment> segs = make_segments(items, 0, req_k);
-    if (segs.empty() && e == cudaSuccess) e = cudaErrorInvalidValue;  // too many units to count
+    if (segs.empty() && !items.empty() && e == cudaSuccess)
+      e = cudaErrorInvalidValue;  // too many units to count
     const size_t ni = items.size();
     const size_t items_off = reqs_off + al(sizeof(ReqDev) * nreq);
     // request table and items go through the pinned mirror
@@ -327,7 +338,7 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
     // the locality sort of each request, then the pack's kernels
     for (int i = 0; i < nreq && e == cudaSuccess; ++i) {
       const ReqRec& R = recs[tickets[i] - 1];
-      if (R.r.nq >= kSortMinQueries)
+      if (R.r.nq >= kSortMinQueries && R.refused == MKNN_OK)
         e = launch_query_sort_any(clouds[R.r.cloud]->dev(), (const float*)(dbase + R.q_off), 3,
                                   R.r.nq, d_hist, (int32_t*)(dbase + R.cell_off),
                                   (int32_t*)(dbase + R.perm_off), s);
@@ -345,6 +356,7 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
     if (e == cudaSuccess) e = cudaEventRecord(sl.t_kern, s);
     for (int i = 0; i < nreq && e == cudaSuccess; ++i) {
       ReqRec& R = recs[tickets[i] - 1];
+      if (R.refused != MKNN_OK) continue;
       const size_t nk = (size_t)R.r.nq * R.r.k * 4;
       void* di = R.out_pinned ? (void*)R.r.out_idx : (void*)(hbase + R.idx_off);
       void* dd = R.out_pinned ? (void*)R.r.out_d2 : (void*)(hbase + R.d2_off);
@@ -352,7 +364,15 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
       if (e == cudaSuccess) e = cudaMemcpyAsync(dd, dbase + R.d2_off, nk, cudaMemcpyDeviceToHost, s);
     }
   }
-  cudaEventRecord(sl.done, s);
+  const cudaError_t de = cudaEventRecord(sl.done, s);
+  if (e == cudaSuccess) e = de;
+  if (e != cudaSuccess) {
+    if (sl.status == MKNN_OK) sl.status = MKNN_ECUDA;
+    // the region is given back next: nothing of the pack may run any more
+    cudaStreamSynchronize(s);
+    for (cudaStream_t a : sl.side.s) cudaStreamSynchronize(a);
+    cudaGetLastError();
+  }
   (void)bytes;
 }
 
