@@ -528,55 +528,6 @@ cudaError_t launch_handover(const ReqDev* d_reqs, Handover* d_ho, int c, int gri
                           0, s);
 }
 
-bool SideStreams::create() {
-  bool ok = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming) == cudaSuccess;
-  for (int i = 0; i < kSideStreams && ok; ++i)
-    ok = cudaStreamCreateWithFlags(&s[i], cudaStreamNonBlocking) == cudaSuccess &&
-         cudaEventCreateWithFlags(&join[i], cudaEventDisableTiming) == cudaSuccess;
-  if (!ok) cudaGetLastError();
-  return ok;
-}
-
-void SideStreams::destroy() {
-  if (fork) cudaEventDestroy(fork);
-  for (int i = 0; i < kSideStreams; ++i) {
-    if (join[i]) cudaEventDestroy(join[i]);
-    if (s[i]) cudaStreamDestroy(s[i]);
-  }
-  *this = SideStreams{};
-}
-
-cudaError_t SideStreams::fork_from(cudaStream_t from, int n) const {
-  if (n <= 0) return cudaSuccess;
-  cudaError_t e = cudaEventRecord(fork, from);
-  for (int i = 0; i < n && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(s[i], fork, 0);
-  return e;
-}
-
-cudaError_t SideStreams::join_to(cudaStream_t from, int n) const {
-  cudaError_t e = cudaSuccess;
-  for (int i = 0; i < n && e == cudaSuccess; ++i) {
-    e = cudaEventRecord(join[i], s[i]);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(from, join[i], 0);
-  }
-  return e;
-}
-
-cudaError_t launch_segments(const ReqDev* d_reqs, const Item* d_items, unsigned* d_next,
-                            const std::vector<Segment>& segs, cudaStream_t s,
-                            const SideStreams& side, int64_t queries) {
-  const bool split = segs.size() > 1 && side.fork && queries <= kSplitMaxQueries;
-  const int nside = split ? (int)std::min<size_t>(kSideStreams, segs.size() - 1) : 0;
-  cudaError_t e = side.fork_from(s, nside);
-  for (size_t i = 0; i < segs.size() && e == cudaSuccess; ++i) {
-    const Segment& g = segs[i];
-    const int on = (int)(i % (size_t)(nside + 1));
-    e = launch_batch_kernel(d_reqs, d_items + g.begin, g.count, g.units, d_next + i, g.launch,
-                            on ? side.s[on - 1] : s);
-  }
-  return e == cudaSuccess ? side.join_to(s, nside) : e;
-}
-
 Mode tuned_mode(int k, int64_t n, int hub) {
   std::lock_guard<std::mutex> lk(g_tune_mu);
   auto it = g_tune.find(TuneKey{k, nbucket_of(n), hub});
@@ -653,20 +604,22 @@ cudaError_t enqueue(mknn_batch* b, cudaStream_t s) {
     e = cudaMemsetAsync(&b->d_ho->count[0], 0, sizeof(Handover) - offsetof(Handover, count), s);
     if (e != cudaSuccess) return e;
   }
-  if ((e = b->side.fork_from(s, b->sorts - 1)) != cudaSuccess) return e;
-  for (int r = 0, i = 0; r < b->nreq; ++r) {
-    if (!b->perm_off[r]) continue;
-    const mknn_batch_req& R = b->reqs[r];
-    const CloudDevHost cd = R.cloud->dev();
-    // the sorts of one stream share its histogram and run one after another
-    const int on = i++ % b->sorts;
-    e = launch_query_sort_split(cd, R.q, R.q_stride, R.nq, (char*)b->d_ws + on * kSortHistBytes,
-                                (int32_t*)((char*)b->d_ws + b->cell_off[r]),
-                                (int32_t*)((char*)b->d_ws + b->perm_off[r]),
-                                on ? b->side.s[on - 1] : s);
-    if (e != cudaSuccess) return e;
-  }
-  if ((e = b->side.join_to(s, b->sorts - 1)) != cudaSuccess) return e;
+  e = b->side.beside(s, b->sorts - 1, [&]() {
+    cudaError_t se = cudaSuccess;
+    for (int r = 0, i = 0; r < b->nreq && se == cudaSuccess; ++r) {
+      if (!b->perm_off[r]) continue;
+      const mknn_batch_req& R = b->reqs[r];
+      // the sorts of one stream share its histogram and run one after another
+      const int on = i++ % b->sorts;
+      se = launch_query_sort_split(R.cloud->dev(), R.q, R.q_stride, R.nq,
+                                   (char*)b->d_ws + on * kSortHistBytes,
+                                   (int32_t*)((char*)b->d_ws + b->cell_off[r]),
+                                   (int32_t*)((char*)b->d_ws + b->perm_off[r]),
+                                   on ? b->side.s[on - 1] : s);
+    }
+    return se;
+  });
+  if (e != cudaSuccess) return e;
   e = launch_segments(b->d_reqs, b->d_items, b->d_next, b->segs, s, b->side, b->total_queries);
   for (int c = 0; c < 3 && e == cudaSuccess; ++c)
     if (b->ho_class[c]) e = launch_handover(b->d_reqs, b->d_ho, c, b->ho_grid[c], s);

@@ -156,8 +156,19 @@ struct SideStreams {
   cudaEvent_t fork = nullptr, join[kSideStreams] = {};
   bool create();   // false when the driver refuses; destroy() is still due
   void destroy();
-  // The first n side streams continue after what is queued on `from`; and
-  // `from` after what is queued on them.
+  // Runs `enqueue` with the first n side streams forked from `from` and joins
+  // them back, also when a call has failed: whoever waits for `from` then
+  // waits for whatever got onto a side stream. Returns the first error.
+  template <class F>
+  cudaError_t beside(cudaStream_t from, int n, F enqueue) const {
+    if (n <= 0) return enqueue();
+    cudaError_t e = fork_from(from, n);
+    if (e == cudaSuccess) e = enqueue();
+    const cudaError_t j = join_to(from, n);
+    return e != cudaSuccess ? e : j;
+  }
+
+ private:
   cudaError_t fork_from(cudaStream_t from, int n) const;
   cudaError_t join_to(cudaStream_t from, int n) const;
 };
