@@ -719,15 +719,15 @@ mknn_status mknn_batch_create(const mknn_batch_req* reqs, int32_t nreq,
   for (int r = 0; r < nreq; ++r) req_k[r] = reqs[r].k;
   int64_t ho_cap[3] = {0, 0, 0};  // queries that may be handed over, per class
   for (int r : orderq) {
+    if (reqs[r].nq == 0) continue;
     const int v = with_trees(variant_index(b->lanes[r], reqs[r].k, b->placement[r]),
                              reqs[r].cloud->trees(reqs[r].k), true);
     if (v == kHandoverVariant || v == kHandoverVariant128) {
       ho_cap[handover_class(reqs[r].k)] += reqs[r].nq;
       b->ho_class[handover_class(reqs[r].k)] = true;
     }
-    if (reqs[r].nq > 0)
-      items.push_back(Item{r, v, 0u, (int32_t)reqs[r].nq,
-                           item_queries(b->lanes[r], rounds, reqs[r].nq)});
+    items.push_back(Item{r, v, 0u, (int32_t)reqs[r].nq,
+                         item_queries(b->lanes[r], rounds, reqs[r].nq)});
   }
   b->segs = make_segments(items, o.blocks_per_sm, req_k);
   if (b->segs.empty() && !items.empty())

@@ -1,0 +1,61 @@
+"""Calls whose kernel is chosen by a rule, where the rule's inputs are unusual."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+import workloads as W
+from paper_2605_02224_gb300 import Cloud
+from paper_2605_02224_gb300 import mknn as M
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def torch():
+    t = pytest.importorskip("torch")
+    if not t.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return t
+
+
+@pytest.fixture(scope="module")
+def patches(torch):
+    """60,000 sites on planar patches (longest list 2,404: box trees)."""
+    P, _ = W.patches4(60_000, 121)
+    c = Cloud.build(P, W.permutation(60_000, 122)).upload()
+    assert c.trees()[0] > 0
+    yield c, P
+    c.close()
+
+
+def _queries(torch, P, nq, seed):
+    lo, hi = W.padded_box(P)
+    return torch.from_numpy(W.box_queries(nq, seed, lo, hi)).cuda()
+
+
+def _request(torch, c, q, k):
+    nq = q.shape[0]
+    return dict(cloud=c.handle, q=q, nq=nq, q_stride=3, k=k,
+                out_idx=torch.full((nq, k), -9, dtype=torch.int32, device="cuda"),
+                out_d2=torch.full((nq, k), -9.0, dtype=torch.float32, device="cuda"))
+
+
+@pytest.mark.parametrize("graph", [0, -1])
+@pytest.mark.parametrize("lanes", [0, 1])
+def test_plan_with_an_empty_request_on_a_cloud_with_trees(torch, patches, graph, lanes):
+    """A request without queries asks for no hand-over, whatever its cloud."""
+    c, _ = patches
+    S, _ = W.sphere(5000, 103)
+    cs = Cloud.build(S, W.permutation(5000, 104)).upload()
+    q = _queries(torch, S, 200_000, 105)
+    full = _request(torch, cs, q, 4)
+    plan = M.mknn_batch_create([full, _request(torch, c, q[:0], 4), _request(torch, c, q[:0], 40)],
+                               lanes=lanes, graph=graph)
+    M.mknn_batch_run(plan, torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    M.mknn_batch_free(plan)
+    idx, d2 = cs.knn(q, 4)
+    torch.cuda.synchronize()
+    assert torch.equal(full["out_idx"], idx) and torch.equal(full["out_d2"], d2)
+    cs.close()
