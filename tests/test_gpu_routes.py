@@ -59,3 +59,50 @@ def test_plan_with_an_empty_request_on_a_cloud_with_trees(torch, patches, graph,
     torch.cuda.synchronize()
     assert torch.equal(full["out_idx"], idx) and torch.equal(full["out_d2"], d2)
     cs.close()
+
+
+@pytest.fixture(scope="module")
+def hubs(torch):
+    """400,000 sites on planar patches: lists of up to about 33,000 entries."""
+    from tests.gpu_util import built_cloud
+    P, _ = W.patches4(400_000, 21200)
+    c = built_cloud(P, W.permutation(400_000, 21201), "patches400k").upload()
+    assert c.trees()[0] > 0 and int(np.diff(c.table()[1]).max()) >= 4096
+    yield c, P
+    c.close()
+
+
+def _ms(torch, run):
+    """The faster of two runs after a first one."""
+    best = float("inf")
+    for rep in range(3):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        run()
+        b.record()
+        b.synchronize()
+        if rep:
+            best = min(best, a.elapsed_time(b))
+    return best
+
+
+@pytest.mark.parametrize("k", [4, 16])
+@pytest.mark.parametrize("option", ["counters", "placement"])
+def test_lanes_of_launches_that_cannot_use_the_trees(torch, hubs, k, option):
+    """A launch that counts, or keeps its lists in registers, reads long lists
+    through; its default is 32 lanes per query there, not one (which takes
+    about thirty times as long), at every number of queries."""
+    c, P = hubs
+    nq = 250_000
+    q = _queries(torch, P, nq, 106)
+    got, want = {}, {}
+    for out, extra in ((got, {}), (want, {"lanes": 32, "placement": 1})):
+        cnt = torch.full((nq, 4), -1, dtype=torch.int32, device="cuda")
+        opt = dict(counters=cnt) if option == "counters" else dict(placement=1)
+        opt.update(extra)
+        out["ms"] = _ms(torch, lambda: out.update(rows=c.knn(q, k, **opt)))
+        out["count"] = cnt
+    for a, b in zip(got["rows"], want["rows"]):
+        assert torch.equal(a, b)
+    assert torch.equal(got["count"], want["count"])
+    assert got["ms"] < 3 * want["ms"], (got["ms"], want["ms"])
