@@ -289,9 +289,11 @@ size_t mknn_knn_workspace_size(int64_t nq, const mknn_knn_opts* opts);
  * One lane per query with the list in shared memory on a cloud with box
  * trees (mknn_cloud_trees): the queries that would read a list with a tree
  * through are handed over to the one-warp kernel (32 lanes, shared memory),
- * which walks the tree; a second launch on the stream, same results. A
- * caller workspace too small for the hand-over (but not for the sort)
- * leaves it out: the lists are then read in rank order. */
+ * which walks the tree; a second launch on the stream, same results. Where
+ * there is no room for the hand-over (a caller workspace that holds the sort
+ * only, no device memory left, a stream being captured before the library
+ * has the scratch for it), the default is one warp per query; with lanes = 1
+ * asked for, the lists are read in rank order. */
 mknn_status mknn_knn_ex(const mknn_cloud* cloud, const float* q, int64_t nq, int32_t q_stride,
                         int32_t k, const int32_t* m, int32_t m_scalar, int32_t* out_idx,
                         float* out_d2, const mknn_knn_opts* opts, mknn_stream_t stream);

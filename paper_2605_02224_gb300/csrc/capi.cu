@@ -140,6 +140,24 @@ cudaError_t scratch_for(cudaStream_t s, size_t bytes, void** out) {
   return cudaSuccess;
 }
 
+// Does the library hold `bytes` of scratch for the stream already?
+bool scratch_holds(cudaStream_t s, size_t bytes) {
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lk(g_scratch_mu);
+  const auto it = g_scratch.find(ScratchKey{dev, s});
+  return it != g_scratch.end() && it->second.second >= bytes;
+}
+
+bool being_captured(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
 size_t perm_bytes(int64_t nq) { return ((size_t)nq * 4 + 255) & ~(size_t)255; }
 
 // Same-manifold queries: the gathered coordinates (float4) and prefix bounds.
@@ -594,7 +612,11 @@ mknn_status mknn_knn_ex(const mknn_cloud* c, const float* q, int64_t nq, int32_t
   cudaStream_t s = (cudaStream_t)stream;
   const int32_t* perm = opts ? opts->order : nullptr;
   // scratch: the sort's (unless an order is given), then the hand-over of
-  // queries to the one-warp kernel (one lane on a cloud with box trees)
+  // queries to the one-warp kernel (one lane on a cloud with box trees). A
+  // call that has no room for the hand-over does without: a caller workspace
+  // too small for it, no device memory, or a stream being captured, where the
+  // library can neither allocate nor, with no sort to hold its scratch for,
+  // should put its address into the graph.
   const size_t sort_need = (!perm && sort_enabled(opts, nq)) ? sort_workspace_bytes(nq) + perm_bytes(nq) : 0;
   const bool wants_defer = trees && lanes == 1 && placement == 2;
   size_t need = sort_need + (wants_defer ? defer_bytes(nq) : 0);
@@ -603,12 +625,22 @@ mknn_status mknn_knn_ex(const mknn_cloud* c, const float* q, int64_t nq, int32_t
     if (opts && opts->workspace) {
       if (opts->workspace_bytes < sort_need)
         return fail(MKNN_EINVAL, "workspace smaller than mknn_knn_workspace_size");
-      if (opts->workspace_bytes < need) need = sort_need;  // too small to hand over: scan instead
+      if (opts->workspace_bytes < need) need = sort_need;
       ws = opts->workspace;
     } else {
-      cudaError_t e = scratch_for(s, need, &ws);
+      if (wants_defer && being_captured(s) &&
+          (!scratch_holds(s, need) || (sort_need == 0 && !(opts && opts->lanes))))
+        need = sort_need;
+      cudaError_t e = need > 0 ? scratch_for(s, need, &ws) : cudaSuccess;
+      if (e != cudaSuccess && need > sort_need) {
+        cudaGetLastError();
+        need = sort_need;
+        e = need > 0 ? scratch_for(s, need, &ws) : cudaSuccess;
+      }
       if (e != cudaSuccess) return fail(MKNN_ENOMEM, "workspace allocation failed");
     }
+    if (wants_defer && need == sort_need && !(opts && opts->lanes))
+      lanes = choose_mode(k, c->n, c->hub_bucket(), nq, trees, false).lanes;
   }
   if (sort_need > 0) {
     int32_t* p = (int32_t*)((char*)ws + sort_workspace_bytes(nq));

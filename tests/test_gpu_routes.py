@@ -106,3 +106,44 @@ def test_lanes_of_launches_that_cannot_use_the_trees(torch, hubs, k, option):
         assert torch.equal(a, b)
     assert torch.equal(got["count"], want["count"])
     assert got["ms"] < 3 * want["ms"], (got["ms"], want["ms"])
+
+
+@pytest.mark.parametrize("k", [4, 16])
+def test_caller_workspace_without_room_for_the_handover(torch, hubs, k):
+    """A workspace that holds the locality sort only: one warp per query, about
+    as fast as when asked for (one lane would read the long lists through)."""
+    c, P = hubs
+    nq = 250_000
+    q = _queries(torch, P, nq, 107)
+    full = M.mknn_knn_workspace_size(nq)
+    bytes_ = full - ((4 * (nq + 64) + 255) & ~255)
+    ws = torch.empty(full, dtype=torch.uint8, device="cuda")
+    want, got = {}, {}
+    for out, opt in ((want, dict(lanes=32, placement=2)),
+                     (got, dict(workspace=ws, workspace_bytes=bytes_))):
+        out["ms"] = _ms(torch, lambda: out.update(rows=c.knn(q, k, **opt)))
+    for a, b in zip(got["rows"], want["rows"]):
+        assert torch.equal(a, b)
+    assert got["ms"] < 2 * want["ms"], (got["ms"], want["ms"])
+
+
+@pytest.mark.parametrize("k", [4, 16])
+def test_captured_call_with_an_order(torch, hubs, k):
+    """A call with its processing order given can be captured on a stream that
+    the library has no scratch for, and the graph gives the call's rows."""
+    c, P = hubs
+    nq = 250_000
+    q = _queries(torch, P, nq, 108)
+    order = torch.empty(nq, dtype=torch.int32, device="cuda")
+    M.mknn_query_order(c.handle, q, nq, 3, order)
+    want = c.knn(q, k)
+    c.knn(q, k, lanes=32, placement=2)
+    idx, d2 = torch.full_like(want[0], -9), torch.full_like(want[1], -9)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        M.mknn_knn_ex(c.handle, q, nq, 3, k, None, 0, idx, d2,
+                      torch.cuda.current_stream().cuda_stream, order=order)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(idx, want[0]) and torch.equal(d2, want[1])
