@@ -292,8 +292,10 @@ size_t mknn_knn_workspace_size(int64_t nq, const mknn_knn_opts* opts);
  * which walks the tree; a second launch on the stream, same results. Where
  * there is no room for the hand-over (a caller workspace that holds the sort
  * only, no device memory left, a stream being captured before the library
- * has the scratch for it), the default is one warp per query; with lanes = 1
- * asked for, the lists are read in rank order. */
+ * has the scratch for it), the default is one warp per query up to a number
+ * of queries that grows with the longest list (about 200,000 at 1,024 entries,
+ * 470,000 at 4,096, 3 million at 32,768); beyond it, and with lanes = 1 asked
+ * for, the lists are read in rank order. */
 mknn_status mknn_knn_ex(const mknn_cloud* cloud, const float* q, int64_t nq, int32_t q_stride,
                         int32_t k, const int32_t* m, int32_t m_scalar, int32_t* out_idx,
                         float* out_d2, const mknn_knn_opts* opts, mknn_stream_t stream);

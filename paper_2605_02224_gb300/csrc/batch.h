@@ -196,10 +196,10 @@ void set_tuned_mode(int k, int64_t n, int hub, Mode m);
 // per query in a launch too small for it.
 // trees: the cloud has box trees and the launch can use them (the one-warp
 // kernel walks them; one lane hands queries that meet them over to it).
-// handover: there is scratch for that hand-over. Without it the launch takes
-// one warp per query, because one lane would read the long lists through
-// (400,000 queries at k = 16 on a 200k-site patch cloud, longest list 34,085:
-// 8.97 ms on one lane without the hand-over, 2.20 ms on one warp).
+// handover: there is scratch for that hand-over. Without it one lane reads the
+// long lists through, so that one warp per query is the faster up to a larger
+// number of queries (400,000 at k = 16 on a 200k-site patch cloud, longest list
+// 34,085: 8.97 ms on one lane without the hand-over, 2.20 ms on one warp).
 Mode choose_mode(int k, int64_t n, int hub, int64_t nq, bool trees = false, bool handover = true);
 
 }  // namespace mknn

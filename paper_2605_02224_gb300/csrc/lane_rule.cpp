@@ -30,8 +30,18 @@ constexpr int kHubBucketWide = 12;
 // Register groups of 4, 8 and 16 lanes are slower than both at every size
 // (100,000 queries, k = 16: 1,638 / 994 / 837 us against 320), so the rule
 // never takes them.
+// On a cloud with trees and no scratch for the hand-over, a lane reads lists of
+// up to 2^(hub + 1) entries through while one warp per query walks the trees.
+// Queries from which one lane is the faster all the same (patch clouds of 20k
+// to 90k sites, k = 1, 4, 16, 32, 40):
+//   longest list 1,100: 135k 155k 175k 180k 205k   1,625: 120k 180k 195k 245k 310k
+//   2,404: 195k 300k 340k 390k 430k   2,695: 275k 340k 280k 270k 280k
+//   3,579: 310k 480k 425k 470k 490k   9,682: 600k 850k 650k 550k 550k
+// (longest 2,695, k = 16, us for one lane / one warp: 150,000 queries 1223 /
+// 704, 300,000 1264 / 1338, 1,000,000 1956 / 4247).
 constexpr int kHubBucketLong = 9;  // a list of 2^9 - 1 entries or more
-int64_t one_lane_min_queries(int k, int hub, bool trees) {
+int64_t one_lane_min_queries(int k, int hub, bool trees, bool handover) {
+  if (trees && !handover) return 102400 + 1100 * (int64_t)k + ((int64_t)90 << hub);
   int64_t q = 40960 + 1100 * (int64_t)k;
   if (k > 32) q += 32768 * (int64_t)(k - 32);
   return (trees || hub >= kHubBucketLong) ? q + 81920 : q;
@@ -43,7 +53,7 @@ Mode choose_mode(int k, int64_t n, int hub, int64_t nq, bool trees, bool handove
   const Mode t = tuned_mode(k, n, hub);
   const int wide = (hub >= kHubBucketWide && !trees) ? 32 : default_lanes(k);
   int lanes = t.lanes ? t.lanes : wide;
-  if (lanes == 1 && (nq < one_lane_min_queries(k, hub, trees) || (trees && !handover))) lanes = 32;
+  if (lanes == 1 && nq < one_lane_min_queries(k, hub, trees, handover)) lanes = 32;
   const int placement = (t.lanes && lanes == t.lanes) ? t.placement : default_placement(k, lanes);
   return Mode{lanes, placement};
 }

@@ -92,10 +92,10 @@ int main() {
   static float q[4], d2[4];
   static int32_t idx[4], order[4];
   uintptr_t stream = 1;  // library scratch is kept per stream: a new one each time
-  for (int hub : {11, 15})
+  for (int hub : {14, 17})
     for (int k : {1, 8, 16, 32, 40, 47, 48, 100}) {
       mknn_cloud* c = cloud(hub, int64_t(1) << hub);
-      const bool trees = k < 48 || hub >= 12, one = k < 48;
+      const bool one = k < 48;  // the trees serve every k
       auto run = [&](mknn_knn_opts o, uintptr_t s) {
         allocs = 0;
         L = mknn::PlainLaunch{};
@@ -110,7 +110,7 @@ int main() {
       mknn_knn_opts o = sorted;
       o.workspace = dev;
       o.workspace_bytes = full;
-      CHECK(run(o, ++stream) == MKNN_OK && L.lanes == (one ? 1 : 32) && !!L.defer == (one && trees) && !allocs);
+      CHECK(run(o, ++stream) == MKNN_OK && L.lanes == (one ? 1 : 32) && !!L.defer == one && !allocs);
       o.workspace_bytes = full - 1;
       CHECK(run(o, ++stream) == MKNN_OK && L.lanes == 32 && L.placement == 2 && !L.defer && !allocs);
       o.workspace_bytes = sort_only;
@@ -143,6 +143,15 @@ int main() {
       capturing = true;
       CHECK(run(sorted, stream) == MKNN_OK && L.lanes == 32 && !L.defer && !allocs);
       capturing = false;
+      // the longer the lists, the more queries it takes until one lane that
+      // reads them through is the faster
+      if (one) {
+        const int64_t line = 102400 + 1100 * k + (int64_t(90) << hub);
+        CHECK(mknn::choose_mode(k, c->n, hub, line - 1, true, false).lanes == 32);
+        CHECK(mknn::choose_mode(k, c->n, hub, line, true, false).lanes == 1);
+        CHECK(mknn::choose_mode(k, c->n, 11, 200000, true, false).lanes == 32);
+        CHECK(mknn::choose_mode(k, c->n, 11, nq, true, false).lanes == 1);
+      }
       if (one) {  // a tuned lane per query follows the same rule
         tuned = mknn::Mode{1, 2};
         o = sorted;
