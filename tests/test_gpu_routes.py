@@ -147,3 +147,20 @@ def test_captured_call_with_an_order(torch, hubs, k):
     g.replay()
     torch.cuda.synchronize()
     assert torch.equal(idx, want[0]) and torch.equal(d2, want[1])
+
+
+@pytest.mark.parametrize("k", [4, 16])
+def test_noalloc_walks_the_trees_of_middling_lists(torch, patches, k):
+    """Longest list 2,404: the no-allocation call takes one warp per query, as
+    fast as the same launch asked for, a little above the number of queries
+    from which one lane (with the hand-over) is mknn_knn's default."""
+    c, P = patches
+    nq = 130_000 + 1100 * k
+    q = _queries(torch, P, nq, 109)
+    want = {}
+    want["ms"] = _ms(torch, lambda: want.update(rows=c.knn(q, k, lanes=32, placement=2)))
+    idx, d2 = (torch.full_like(a, -9) for a in want["rows"])
+    ms = _ms(torch, lambda: M.mknn_knn_noalloc(c.handle, q, nq, 3, k, None, 0, idx, d2,
+                                               torch.cuda.current_stream().cuda_stream))
+    assert torch.equal(idx, want["rows"][0]) and torch.equal(d2, want["rows"][1])
+    assert ms < 1.4 * want["ms"], (ms, want["ms"])
