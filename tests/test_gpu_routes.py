@@ -164,3 +164,49 @@ def test_noalloc_walks_the_trees_of_middling_lists(torch, patches, k):
                                                torch.cuda.current_stream().cuda_stream))
     assert torch.equal(idx, want["rows"][0]) and torch.equal(d2, want["rows"][1])
     assert ms < 1.4 * want["ms"], (ms, want["ms"])
+
+
+@pytest.mark.parametrize("lanes", [0, 1, 8, 32])
+def test_plan_of_many_requests(torch, patches, lanes):
+    """Thousands of requests of 0 to 70 queries in each segment, in an order of
+    sizes that leaves whole runs of one-unit requests to a warp: every row is
+    the row of one launch over all queries."""
+    c, P = patches
+    rng = np.random.default_rng(110)
+    sizes = np.concatenate([rng.integers(0, 71, 1500), np.ones(2500, int), rng.integers(0, 9, 500)])
+    q = _queries(torch, P, int(sizes.sum()), 111)
+    ends = np.cumsum(sizes)
+    reqs, out = [], {}
+    for k in (5, 20):
+        out[k] = [torch.full((len(q), k), -9, dtype=torch.int32, device="cuda"),
+                  torch.full((len(q), k), -9.0, dtype=torch.float32, device="cuda")]
+        for e, s in zip(ends, sizes):
+            a = int(e - s)
+            reqs.append(dict(cloud=c.handle, q=q[a:], nq=int(s), q_stride=3, k=k,
+                             out_idx=out[k][0][a:], out_d2=out[k][1][a:]))
+    plan = M.mknn_batch_create(reqs, lanes=lanes)
+    for _ in range(2):
+        M.mknn_batch_run(plan, torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    M.mknn_batch_free(plan)
+    for k in (5, 20):
+        want = c.knn(q, k)
+        assert torch.equal(out[k][0], want[0]) and torch.equal(out[k][1], want[1])
+
+
+def test_plan_of_many_requests_costs_about_one_request(torch):
+    """20,000 requests of 16 queries against one request of all of them."""
+    P, _ = W.torus(100_000, 112)
+    c = Cloud.build(P, W.permutation(100_000, 113)).upload()
+    q = _queries(torch, P, 320_000, 114)
+    ms = []
+    for n in (1, 20_000):
+        whole = _request(torch, c, q, 8)
+        per = 320_000 // n
+        reqs = [dict(whole, q=q[j * per:], nq=per, out_idx=whole["out_idx"][j * per:],
+                     out_d2=whole["out_d2"][j * per:]) for j in range(n)]
+        plan = M.mknn_batch_create(reqs, lanes=32, sort=-1)
+        ms.append(_ms(torch, lambda: M.mknn_batch_run(plan, torch.cuda.current_stream().cuda_stream)))
+        M.mknn_batch_free(plan)
+    assert ms[1] < 1.6 * ms[0], ms
+    c.close()
