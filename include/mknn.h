@@ -430,8 +430,8 @@ mknn_status mknn_knn_batch(const mknn_batch_req* reqs, int32_t nreq, const mknn_
  * warm-up) on max(sample, 2 x SMs x 2048) queries of that request (tiled
  * when it has fewer); the fastest (lanes, placement) goes into the
  * process-wide tuning table. Plans, plain launches and the server take the
- * table's entry, one warp per query where it says one lane and the launch is
- * too small for that. If the environment variable MKNN_TUNE_LOG
+ * table's entry, one warp per query where it says fewer than 32 lanes and the
+ * launch is too small for one lane. If the environment variable MKNN_TUNE_LOG
  * names a file, one line per timed candidate (k, n, hub bucket, sample,
  * lanes, placement, ms) is appended to it. Synchronises the stream.
  * Errors: EINVAL, ENOMEM, ECUDA. */

@@ -192,8 +192,8 @@ cudaError_t launch_segments(const ReqDev* d_reqs, const Item* d_items, unsigned*
 Mode tuned_mode(int k, int64_t n, int hub);
 void set_tuned_mode(int k, int64_t n, int hub, Mode m);
 // Mode for a launch of nq queries: the tuned (or default) lanes for
-// (k, n, hub) and their placement; one lane per query turns into one warp
-// per query in a launch too small for it.
+// (k, n, hub) and their placement; fewer than 32 lanes turn into one warp
+// per query in a launch too small for one lane.
 // trees: the cloud has box trees and the launch can use them (the one-warp
 // kernel walks them; one lane hands queries that meet them over to it).
 // handover: there is scratch for that hand-over. Without it one lane reads the

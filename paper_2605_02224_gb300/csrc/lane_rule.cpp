@@ -53,7 +53,11 @@ Mode choose_mode(int k, int64_t n, int hub, int64_t nq, bool trees, bool handove
   const Mode t = tuned_mode(k, n, hub);
   const int wide = (hub >= kHubBucketWide && !trees) ? 32 : default_lanes(k);
   int lanes = t.lanes ? t.lanes : wide;
-  if (lanes == 1 && nq < one_lane_min_queries(k, hub, trees, handover)) lanes = 32;
+  // a table made by an earlier tuner may hold register groups: slower than
+  // one warp per query in a small launch (100k-site torus, k = 8, 4 / 8 / 16
+  // lanes: 64 queries 205 / 90 / 51 us against 21, 10,000 259 / 132 / 79
+  // against 57)
+  if (lanes < 32 && nq < one_lane_min_queries(k, hub, trees, handover)) lanes = 32;
   const int placement = (t.lanes && lanes == t.lanes) ? t.placement : default_placement(k, lanes);
   return Mode{lanes, placement};
 }

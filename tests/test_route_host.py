@@ -184,3 +184,33 @@ def _run(tmp_path, main):
 
 def test_no_room_for_the_handover_means_one_warp_per_query(tmp_path):
     _run(tmp_path, MAIN_ROOM)
+
+
+MAIN_TUNED = r"""
+int main() {
+  // a tuned width below 32 lanes serves large launches; small ones take one
+  // warp per query
+  for (int lanes : {1, 4, 8, 16})
+    for (int k : {1, 8, 16}) {
+      tuned = mknn::Mode{lanes, lanes == 1 ? 2 : 1};
+      for (int64_t nq : {1, 64, 1000, 10000, 40000}) {
+        const mknn::Mode m = mknn::choose_mode(k, 100000, 8, nq, false);
+        L.k = k;
+        L.lanes = m.lanes;
+        CHECK(m.lanes == 32 && m.placement == 2);
+      }
+      const mknn::Mode m = mknn::choose_mode(k, 100000, 8, 1 << 20, false);
+      CHECK(m.lanes == tuned.lanes && m.placement == tuned.placement);
+    }
+  tuned = mknn::Mode{32, 1};  // registers, when tuned so, at every size
+  for (int64_t nq : {64, 1 << 20}) {
+    const mknn::Mode m = mknn::choose_mode(8, 100000, 8, nq, false);
+    CHECK(m.lanes == 32 && m.placement == 1);
+  }
+  std::printf("ok\n");
+}
+"""
+
+
+def test_tuned_widths_of_small_launches(tmp_path):
+    _run(tmp_path, MAIN_TUNED)
