@@ -238,8 +238,9 @@ typedef struct {
                            up, in batches below about 41,000 + 1,100 k
                            queries - 82,000 more on clouds with long
                            successor lists, 33,000 more for each k above
-                           32 - and on clouds with very long lists and
-                           no box trees; else 1), or
+                           32; on 152 SMs, in proportion on others - and
+                           on clouds with very long lists and no box
+                           trees; else 1), or
                            1, 4, 8, 16, 32 (4 and 8 hold k <= 64; one
                            lane above 64 needs placement 2 and no
                            counters) */

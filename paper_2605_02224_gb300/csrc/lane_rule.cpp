@@ -14,7 +14,8 @@ constexpr int kHubBucketWide = 12;
 // Queries of one launch from which one lane per query is faster than one
 // warp per query. One lane per query takes about the time of its longest
 // query whatever the number of queries, until they fill the GPU; one warp
-// per query takes time in proportion to it. On a 300k-site torus (queries
+// per query takes time in proportion to it, so the line grows with the number
+// of SMs; the figures are of 152. On a 300k-site torus (queries
 // half in the box, half near the surface; us for one lane / one warp per
 // query at 40,000 and 80,000 queries, the locality sort included):
 //   k = 1: 102 / 102, 103 / 163     k = 8: 184 / 159, 198 / 277
@@ -41,10 +42,14 @@ constexpr int kHubBucketWide = 12;
 // 704, 300,000 1264 / 1338, 1,000,000 1956 / 4247).
 constexpr int kHubBucketLong = 9;  // a list of 2^9 - 1 entries or more
 int64_t one_lane_min_queries(int k, int hub, bool trees, bool handover) {
-  if (trees && !handover) return 102400 + 1100 * (int64_t)k + ((int64_t)90 << hub);
   int64_t q = 40960 + 1100 * (int64_t)k;
-  if (k > 32) q += 32768 * (int64_t)(k - 32);
-  return (trees || hub >= kHubBucketLong) ? q + 81920 : q;
+  if (trees && !handover) {
+    q += 61440 + ((int64_t)90 << hub);
+  } else {
+    if (k > 32) q += 32768 * (int64_t)(k - 32);
+    if (trees || hub >= kHubBucketLong) q += 81920;
+  }
+  return q * num_sms() / 152;
 }
 
 }  // namespace

@@ -62,7 +62,8 @@ Mode tuned_mode(int, int64_t, int) { return tuned; }
 int default_lanes(int k) { return k >= kWarpMinK ? 32 : 1; }
 int default_placement(int, int lanes) { return lanes == 1 || lanes == 32 ? 2 : 1; }
 int plain_max_k(int lanes) { return lanes == 4 || lanes == 8 ? 64 : 128; }
-int num_sms() { return 152; }
+static int sms = 152;
+int num_sms() { return sms; }
 size_t sort_workspace_bytes(int64_t nq) { return kSortHistBytes + (((size_t)nq * 4 + 255) & ~(size_t)255); }
 static cudaError_t launched() { return cudaGetLastError(); }  // as the launchers return it
 cudaError_t launch_query_sort(const CloudDevHost&, const float*, int32_t, int64_t, void*, int32_t*, cudaStream_t) { return launched(); }
@@ -214,3 +215,27 @@ int main() {
 
 def test_tuned_widths_of_small_launches(tmp_path):
     _run(tmp_path, MAIN_TUNED)
+
+
+MAIN_SMS = r"""
+int main() {
+  // the number of queries from which one lane is the default, on a GPU and on
+  // half of one: 40,960 + 1,100 k, more with long lists and above k = 32
+  for (int part : {1, 2})
+    for (int k : {1, 16, 32, 33, 47})
+      for (int hub : {8, 9, 12}) {
+        mknn::sms = 152 / part;
+        const bool trees = hub == 12;
+        const int64_t line = (40960 + 1100 * k + (k > 32 ? 32768 * (k - 32) : 0) +
+                              (hub >= 9 ? 81920 : 0)) / part;
+        L.k = k;
+        CHECK(mknn::choose_mode(k, 100000, hub, line - 1, trees).lanes == 32);
+        CHECK(mknn::choose_mode(k, 100000, hub, line, trees).lanes == 1);
+      }
+  std::printf("ok\n");
+}
+"""
+
+
+def test_one_lane_line_follows_the_number_of_sms(tmp_path):
+    _run(tmp_path, MAIN_SMS)
