@@ -70,7 +70,7 @@ mknn_status mknn_knn_ex(const mknn_cloud*, const float*, int64_t nq, int32_t, in
 
 namespace mknn {
 void set_error(const std::string&) {}
-Mode choose_mode(int, int64_t, int, int64_t, bool) { return Mode{32, 2}; }
+Mode choose_mode(int, int64_t, int, int64_t, bool, bool) { return Mode{32, 2}; }
 int default_placement(int, int lanes) { return lanes == 4 ? 1 : 2; }
 int variant_index(int lanes, int k, int) { return lanes == 4 ? (k <= 64 ? 2 : -1) : 16; }
 std::vector<Segment> make_segments(std::vector<Item>& items, int, const std::vector<int>&) {
