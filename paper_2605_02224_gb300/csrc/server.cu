@@ -95,6 +95,7 @@ class Arena {
 
 struct ReqRec {
   mknn_request r;
+  const mknn_cloud* cloud = nullptr;
   Clock::time_point t_submit, t_done;
   int32_t state = 0;  // 0 pending, 1 done, <0 failed
   bool q_pinned = false, out_pinned = false;
@@ -112,7 +113,10 @@ struct Slot {
   cudaEvent_t t0 = nullptr, t_h2d = nullptr, t_kern = nullptr;
   bool busy = false;
   mknn_status status = MKNN_OK;  // of the launch: what its requests end with
+  // the pack's requests, looked up under the lock: submit and add_cloud grow
+  // the server's tables while a pack is launched
   std::vector<uint64_t> tickets;
+  std::vector<ReqRec*> reqs;
   size_t off = 0, bytes = 0;
 };
 
@@ -169,7 +173,7 @@ struct mknn_server {
 
   void run();
   void reap_locked();
-  void launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, size_t bytes);
+  void launch(Slot& sl);
 };
 
 void mknn_server::reap_locked() {
@@ -181,8 +185,9 @@ void mknn_server::reap_locked() {
       cudaGetLastError();
       if (sl.status == MKNN_OK) sl.status = MKNN_ECUDA;
     }
-    for (uint64_t t : sl.tickets) {
-      ReqRec& R = recs[t - 1];
+    for (size_t i = 0; i < sl.tickets.size(); ++i) {
+      const uint64_t t = sl.tickets[i];
+      ReqRec& R = *sl.reqs[i];
       const mknn_status st = sl.status != MKNN_OK ? sl.status : R.refused;
       if (st == MKNN_OK) {
         if (!R.out_pinned) {
@@ -216,6 +221,7 @@ void mknn_server::reap_locked() {
     arena.release(sl.off, sl.bytes);
     sl.busy = false;
     sl.tickets.clear();
+    sl.reqs.clear();
     --inflight;
   }
   cv_done.notify_all();
@@ -223,15 +229,15 @@ void mknn_server::reap_locked() {
 
 // Issues one pack on a slot (called without the lock held). What goes wrong
 // is the slot's status, which its requests end with.
-void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, size_t bytes) {
+void mknn_server::launch(Slot& sl) {
   cudaStream_t s = sl.s;
-  char* dbase = d_arena + off;
-  char* hbase = h_arena + off;
+  char* dbase = d_arena + sl.off;
+  char* hbase = h_arena + sl.off;
   cudaError_t e = cudaEventRecord(sl.t0, s);
   sl.status = MKNN_OK;
   if (o.plain) {
     // baseline: the request alone through the plain entry point
-    ReqRec& R = recs[tickets[0] - 1];
+    ReqRec& R = *sl.reqs[0];
     const mknn_request& q = R.r;
     const size_t qb = (size_t)q.nq * 12, nk = (size_t)q.nq * q.k * 4;
     const void* src = q.q;
@@ -246,7 +252,7 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
     ko.workspace = dbase + R.cell_off;
     ko.workspace_bytes = al((size_t)q.nq * 4) * 2 + kSortHistBytes;
     if (e == cudaSuccess)
-      sl.status = mknn_knn_ex(clouds[q.cloud], (const float*)(dbase + R.q_off), q.nq, 3, q.k,
+      sl.status = mknn_knn_ex(R.cloud, (const float*)(dbase + R.q_off), q.nq, 3, q.k,
                               nullptr, q.m, (int32_t*)(dbase + R.idx_off),
                               (float*)(dbase + R.d2_off), &ko, (mknn_stream_t)s);
     if (sl.status != MKNN_OK) e = cudaErrorLaunchFailure;  // nothing to copy back
@@ -260,16 +266,16 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
     unsigned* d_next = (unsigned*)dbase;
     void* d_hist = dbase + 256;
     const size_t reqs_off = 256 + kSortHistBytes;
-    const int nreq = (int)tickets.size();
+    const int nreq = (int)sl.reqs.size();
     std::vector<ReqDev> rd(nreq);
     std::vector<Item> items;
     std::vector<int> req_k(nreq);
     int64_t pack_nq = 0;  // the pack runs as one launch per variant: its size sets the lanes
-    for (int i = 0; i < nreq; ++i) pack_nq += recs[tickets[i] - 1].r.nq;
+    for (const ReqRec* R : sl.reqs) pack_nq += R->r.nq;
     std::vector<int> lanes(nreq), placement(nreq);
     for (int i = 0; i < nreq; ++i) {
-      const mknn_request& q = recs[tickets[i] - 1].r;
-      const mknn_cloud* c = clouds[q.cloud];
+      const mknn_request& q = sl.reqs[i]->r;
+      const mknn_cloud* c = sl.reqs[i]->cloud;
       const Mode chosen = choose_mode(q.k, c->n, c->hub_bucket(), pack_nq, c->trees(q.k));
       lanes[i] = o.lanes ? o.lanes : chosen.lanes;
       placement[i] = o.lanes ? default_placement(q.k, lanes[i]) : chosen.placement;
@@ -279,9 +285,9 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
     int2* d_pairs = (int2*)(dbase + ho_off + al(sizeof(Handover)));
     int64_t ho_cap[3] = {0, 0, 0};
     for (int i = 0; i < nreq; ++i) {
-      ReqRec& R = recs[tickets[i] - 1];
+      ReqRec& R = *sl.reqs[i];
       const mknn_request& q = R.r;
-      const mknn_cloud* c = clouds[q.cloud];
+      const mknn_cloud* c = R.cloud;
       const int base = variant_index(lanes[i], q.k, placement[i]);
       if (base < 0) {  // k above what the server's lanes hold: the others go without it
         R.refused = MKNN_EINVAL;
@@ -337,9 +343,9 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
     if (e == cudaSuccess) e = cudaEventRecord(sl.t_h2d, s);
     // the locality sort of each request, then the pack's kernels
     for (int i = 0; i < nreq && e == cudaSuccess; ++i) {
-      const ReqRec& R = recs[tickets[i] - 1];
+      const ReqRec& R = *sl.reqs[i];
       if (R.r.nq >= kSortMinQueries && R.refused == MKNN_OK)
-        e = launch_query_sort_any(clouds[R.r.cloud]->dev(), (const float*)(dbase + R.q_off), 3,
+        e = launch_query_sort_any(R.cloud->dev(), (const float*)(dbase + R.q_off), 3,
                                   R.r.nq, d_hist, (int32_t*)(dbase + R.cell_off),
                                   (int32_t*)(dbase + R.perm_off), s);
     }
@@ -355,7 +361,7 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
         e = launch_handover((const ReqDev*)(dbase + reqs_off), d_ho, c, handover_grid(c), s);
     if (e == cudaSuccess) e = cudaEventRecord(sl.t_kern, s);
     for (int i = 0; i < nreq && e == cudaSuccess; ++i) {
-      ReqRec& R = recs[tickets[i] - 1];
+      ReqRec& R = *sl.reqs[i];
       if (R.refused != MKNN_OK) continue;
       const size_t nk = (size_t)R.r.nq * R.r.k * 4;
       void* di = R.out_pinned ? (void*)R.r.out_idx : (void*)(hbase + R.idx_off);
@@ -373,7 +379,6 @@ void mknn_server::launch(Slot& sl, std::vector<uint64_t>& tickets, size_t off, s
     for (cudaStream_t a : sl.side.s) cudaStreamSynchronize(a);
     cudaGetLastError();
   }
-  (void)bytes;
 }
 
 void mknn_server::run() {
@@ -454,13 +459,14 @@ void mknn_server::run() {
     }
     free_slot->busy = true;
     free_slot->tickets = take;
+    for (uint64_t t : take) free_slot->reqs.push_back(&recs[t - 1]);
     free_slot->off = off;
     free_slot->bytes = bytes;
     ++inflight;
     ++launches;
     packed += (int64_t)take.size();
     lk.unlock();
-    launch(*free_slot, free_slot->tickets, off, bytes);
+    launch(*free_slot);
     lk.lock();
   }
 }
@@ -543,6 +549,7 @@ mknn_status mknn_server_submit(mknn_server* s, const mknn_request* r, uint64_t* 
   lk.lock();
   ReqRec R;
   R.r = *r;
+  R.cloud = c;
   R.q_pinned = qp;
   R.out_pinned = op;
   R.t_submit = Clock::now();

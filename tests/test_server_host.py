@@ -207,3 +207,43 @@ def _run(tmp_path, main, *flags):
 
 def test_requests_of_a_failed_launch_fail(tmp_path):
     _run(tmp_path, MAIN_ERRORS)
+
+
+MAIN_THREADS = r"""
+int main() {
+  mknn_cloud c;
+  c.n = 1000;
+  c.rowp.assign(1001, 0);
+  for (int plain = 0; plain < 2; ++plain) {
+    mknn_server* s = server(&c, plain, 0);
+    std::vector<std::vector<Req>> reqs(3, std::vector<Req>(400));
+    std::vector<std::thread> th;
+    for (int t = 0; t < 3; ++t)
+      th.emplace_back([&, t] {
+        for (int i = 0; i < 400; ++i) {
+          int32_t id = 0;
+          if (t == 0 && i % 4 == 0) CHECK(mknn_server_add_cloud(s, &c, &id) == MKNN_OK);
+          submit(s, reqs[t][i], 1 + i % 7, 1 + (i + t) % 32, id);
+        }
+      });
+    for (auto& t : th) t.join();
+    CHECK(mknn_server_drain(s, 60.0) == MKNN_OK);
+    for (auto& v : reqs)
+      for (Req& r : v) CHECK(state(s, r) == 1 && all(r, r.k));
+    CHECK(mknn_server_destroy(s, 10.0) == MKNN_OK);
+  }
+  std::printf("ok\n");
+}
+"""
+
+
+def test_submitting_while_packs_are_launched(tmp_path):
+    """Threads that submit requests and add clouds while the scheduler thread
+    launches packs: no data race (ThreadSanitizer) and every row is right."""
+    probe = tmp_path / "p.cpp"
+    probe.write_text("int main() {}")
+    built = subprocess.run(["g++", "-fsanitize=thread", str(probe), "-o", str(tmp_path / "p")],
+                           capture_output=True)
+    if built.returncode or subprocess.run([str(tmp_path / "p")], capture_output=True).returncode:
+        pytest.skip("no ThreadSanitizer")
+    _run(tmp_path, MAIN_THREADS, "-fsanitize=thread", "-g")
