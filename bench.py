@@ -100,12 +100,22 @@ def _peaks():
 WARP_MIN_K = 48   # from this k the library's default is one warp per query
 
 
-def _query_kernel_name(lanes: int, k: int, placement: int, trees: bool = False) -> str:
-    """The query kernel a plain launch with these options runs (its default:
-    one lane per query with the list in shared memory, one warp per query
-    with the warp's list in shared memory from k = 48; the one-warp kernel's
-    second form walks the box trees of a cloud that has them)."""
-    if (lanes == 0 and k >= WARP_MIN_K) or (lanes == 32 and placement in (0, 2)):
+def _one_lane_min_queries(k: int) -> int:
+    """Queries of a launch from which one lane per query is the default below
+    k = 48, on a cloud without long lists, on 152 SMs."""
+    return 40960 + 1100 * k + 32768 * max(0, k - 32)
+
+
+def _query_kernel_name(lanes: int, k: int, placement: int, trees: bool = False,
+                       nq: int | None = None) -> str:
+    """The query kernel a plain launch of nq queries (None: a large one) with
+    these options runs (its default: one lane per query with the list in shared
+    memory, one warp per query with the warp's list in shared memory from k = 48
+    and in small launches; the one-warp kernel's second form walks the box trees
+    of a cloud that has them)."""
+    if lanes == 0 and (k >= WARP_MIN_K or (nq is not None and nq < _one_lane_min_queries(k))):
+        lanes = 32
+    if lanes == 32 and placement in (0, 2):
         kc = 32 if k <= 32 else (64 if k <= 64 else 128)
         return f"knn_plain_warp_kernel<{kc}, {'true' if trees else 'false'}>"
     if lanes in (0, 1) and placement in (0, 2):
@@ -790,7 +800,7 @@ def prefix_section(args, M, torch, built=None):
         "workload": f"bumpy sphere n={wl.n}, {nq} queries (half volume, half near-surface), "
                     f"m log-uniform in [1000, n] per query, k={k}",
         "value": nq / (t / 1e3), "unit": UNIT, "ms_per_step": t, "steps": args.steps,
-        "roofline": _roofline(alg, t, nq, l2=args._l2, kernel=_query_kernel_name(0, k, 0),
+        "roofline": _roofline(alg, t, nq, l2=args._l2, kernel=_query_kernel_name(0, k, 0, nq=nq),
                               counts={"rows": rows / nq, "entries": entries / nq,
                                       "coords": coords / nq, "transitions": trans / nq}),
         "config": {"E": cloud.stats()["entries"], "l2": "flushed before every timed step",
@@ -840,7 +850,7 @@ def sites_section(args, M, torch, cloud, n):
         out[f"k{k}"] = {"workload": f"torus n={n}, {n} site queries ({mode}), k={k}",
                         "value": n / (t / 1e3), "unit": UNIT, "ms_per_step": t,
                         "roofline": _roofline(alg, t, n, l2=args._l2,
-                                              kernel=_query_kernel_name(0, k, 0),
+                                              kernel=_query_kernel_name(0, k, 0, nq=n),
                                               counts={"rows": rows / n, "entries": entries / n,
                                                       "coords": coords / n,
                                                       "transitions": trans / n}),
@@ -1241,7 +1251,7 @@ def main():
     khash = _kernel_hash()
     rec = _profile_record(khash)
     roof = _roofline(alg_bytes, kern_s * 1e3, nq, l2=args._l2, rec=rec,
-                     kernel=_query_kernel_name(lanes, k, args.placement),
+                     kernel=_query_kernel_name(lanes, k, args.placement, nq=nq),
                      counts={"rows": rows / nq, "entries": entries / nq, "coords": coords / nq,
                              "transitions": trans / nq})
     roof["traffic"] = _profiled_traffic(khash, wl.n, nq)
@@ -1258,7 +1268,8 @@ def main():
         no_sort = {"value": nq / (t_ns / 1e3), "unit": UNIT, "ms_per_step": t_ns,
                    "speedup_of_sort": t_ns / ms_per_step,
                    "roofline": _roofline(alg_bytes, t_ns, nq, l2=args._l2,
-                                         kernel=_query_kernel_name(lanes, k, args.placement)),
+                                         kernel=_query_kernel_name(lanes, k, args.placement,
+                                                                   nq=nq)),
                    "clocks": clk_ns}
         # k sweep on the same cloud and queries
         k_sweep = []
@@ -1274,7 +1285,7 @@ def main():
             k_sweep.append({"k": kk, "value": nq / (t_k / 1e3), "unit": UNIT, "ms_per_step": t_k,
                             "roofline": _roofline(_alg_bytes(r_, e_, c_, nq, kk), t_k, nq,
                                                   l2=args._l2,
-                                                  kernel=_query_kernel_name(lanes, kk, 0),
+                                                  kernel=_query_kernel_name(lanes, kk, 0, nq=nq),
                                                   counts={"rows": r_ / nq, "entries": e_ / nq,
                                                           "coords": c_ / nq,
                                                           "transitions": t_ / nq}),

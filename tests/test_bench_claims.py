@@ -168,3 +168,17 @@ def test_oracle_pool_rate_on_a_tiny_sample():
     Q = W.box_queries(200, 4, [-1.5] * 3, [1.5] * 3)
     rate, s, dt, cores = bench.oracle_rate(P, Q, 4, 0.2, cores=2)
     assert cores == 2 and 4 <= s <= 196 and rate > 0 and dt > 0
+
+
+def test_query_kernel_name_of_small_launches():
+    """Below the number of queries from which one lane is the default, the
+    kernel named is the one-warp kernel; the line is the library's."""
+    src = _read("lane_rule.cpp")
+    assert "int64_t q = 40960 + 1100 * (int64_t)k;" in src
+    assert "if (k > 32) q += 32768 * (int64_t)(k - 32);" in src
+    for k, kc, one in ((16, 32, "<256, 1, 16, false>"), (40, 64, "<128, 2, 0, false>")):
+        line = bench._one_lane_min_queries(k)
+        assert bench._query_kernel_name(0, k, 0, nq=line - 1) == f"knn_plain_warp_kernel<{kc}, false>"
+        assert bench._query_kernel_name(0, k, 0, nq=line) == f"knn_plain_smem_kernel{one}"
+    assert bench._query_kernel_name(1, 16, 0, nq=10) == "knn_plain_smem_kernel<256, 1, 16, false>"
+    assert bench._query_kernel_name(0, 16, 1, nq=10) == "knn_plain_kernel<32, S>"
