@@ -210,3 +210,47 @@ def test_plan_of_many_requests_costs_about_one_request(torch):
         M.mknn_batch_free(plan)
     assert ms[1] < 1.6 * ms[0], ms
     c.close()
+
+
+@pytest.mark.parametrize("trees", [False, True])
+@pytest.mark.parametrize("k", [8, 33, 34])
+def test_default_lanes_on_both_sides_of_the_line(torch, patches, trees, k):
+    """The number of queries from which one lane is the default, above k = 32
+    too: a plan's lanes on both sides of it, and its rows and the plain
+    launch's against one warp per query in registers."""
+    if trees:
+        c, P = patches
+    else:
+        P, _ = W.torus(4000, 115)
+        c = Cloud.build(P, W.permutation(4000, 116)).upload()
+        assert int(np.diff(c.table()[1]).max()) < 511
+    line = 40960 + 1100 * k + 32768 * max(0, k - 32) + (81920 if trees else 0)
+    line = line * torch.cuda.get_device_properties(0).multi_processor_count // 152
+    for nq, lanes in ((line - 1, 32), (line, 1)):
+        q = _queries(torch, P, nq, 117)
+        r = _request(torch, c, q, k)
+        plan = M.mknn_batch_create([r])
+        assert M.mknn_batch_info(plan, 1)[0].tolist() == [lanes]
+        M.mknn_batch_run(plan, torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        M.mknn_batch_free(plan)
+        want = c.knn(q, k, lanes=32, placement=1)
+        for got in ((r["out_idx"], r["out_d2"]), c.knn(q, k)):
+            assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    if not trees:
+        c.close()
+
+
+def test_large_plan_with_several_segments(torch, patches):
+    """More queries than segments are run side by side for: one after another
+    on the caller's stream, the hand-over after them."""
+    c, P = patches
+    q = _queries(torch, P, 1_100_000, 118)
+    reqs = [_request(torch, c, q, k) for k in (2, 12)]
+    plan = M.mknn_batch_create(reqs)
+    M.mknn_batch_run(plan, torch.cuda.current_stream().cuda_stream)
+    torch.cuda.synchronize()
+    M.mknn_batch_free(plan)
+    for r in reqs:
+        want = c.knn(q, r["k"], lanes=32, placement=2)
+        assert torch.equal(r["out_idx"], want[0]) and torch.equal(r["out_d2"], want[1])
