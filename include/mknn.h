@@ -361,9 +361,9 @@ mknn_status mknn_cloud_check(const mknn_cloud* cloud, int32_t* flags);
 
 /* ------------------------------------------------------- batched queries
  * Many requests, each on its own cloud with its own k and m, answered by
- * persistent kernel launches, one per kernel variant present, each draining
- * its own device work queue (items of a few rounds of one request's
- * queries). Per request the kernel variant
+ * persistent kernel launches, one per kernel variant and list class present,
+ * each draining its own device work queue (units of one round of a request's
+ * queries, one per lane group of a warp). Per request the kernel variant
  * (lanes per query, candidate slots) comes from the tuning table, filled by
  * mknn_batch_tune, or a default. A plan captures its launches (query
  * locality sorts + the persistent kernel) in a CUDA graph and replays it.

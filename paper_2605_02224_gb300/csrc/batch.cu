@@ -5,13 +5,14 @@
 // A plan covers many requests, each (cloud, queries, k, m, outputs). Every
 // request is served by the kernel variant (lanes per query G, candidate
 // slots per lane S) the tuner chose for its (k, cloud size, cloud shape),
-// and cut into work items of a few rounds of its group width. The items of
-// each variant form one queue, drained by one persistent launch of that
-// variant's kernel (SM count x resident blocks): each warp takes the next
-// item with one atomic. Items of one request are contiguous in a queue, so
-// the warps working at any moment share one cloud's table in L2; requests
-// are queued by decreasing estimated cost so that a queue ends with short
-// items. The segments of a small plan run side by side on a few streams.
+// and cut into work units of one round of its group width. The requests of
+// each variant and list class form a segment, drained by one persistent launch
+// of that variant's kernel (SM count x resident blocks): each warp takes the
+// next unit's number with one atomic and finds its request in the segment's
+// table. Units of one request have consecutive numbers, so the warps working
+// at any moment share one cloud's table in L2; requests are queued by
+// decreasing estimated cost so that a segment ends with short units. The
+// segments of a small plan run side by side on a few streams.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -672,6 +673,7 @@ mknn_status mknn_batch_create(const mknn_batch_req* reqs, int32_t nreq,
     b->sorts = std::max(1, std::min(sorted, kSideStreams + 1));
   }
   size_t off = b->sorts * kSortHistBytes;
+  static_assert(kSortMinQueries == 4096, "the line of the loop below");
   for (int r = 0; r < nreq; ++r) {
     if (!sort_on || reqs[r].nq < (o.sort > 0 ? 1 : 4096)) continue;
     b->cell_off[r] = off;

@@ -1365,6 +1365,15 @@ __host__ __device__ constexpr int kWarpListWords(int kc) { return kc + kHubStack
 // 2402, 64 queries 105 / 125; on a 300k-site torus 100,000 queries at k = 64
 // 1532 / 1348, at k = 16 550 / 477, 64 queries the same; with trees, k = 32,
 // 10,000 queries 276 / 292, 60,000 609 / 546.
+// The bound costs spills (ptxas -v: 0 to 68 bytes in the plain kernels, 52 to
+// 192 in the persistent and hand-over kernels, which keep the request too);
+// left alone the latter take 64 to 104 registers and are slower but for small
+// launches with trees. Plans on a 300k-site torus, us held / left alone:
+// 20,000 queries at k = 8 88 / 92, k = 64 346 / 425, k = 128 721 / 826; 300,000
+// at k = 32 on one warp each 2005 / 2188, k = 64 4027 / 5146, k = 100 7165 /
+// 8350; on a 200k-site patch cloud with trees 20,000 at k = 8 202 / 189, k = 32
+// 302 / 283, k = 100 802 / 1072; 60,000 at k = 32 605 / 715; 300,000 at k = 100
+// 9958 / 13872; with the hand-over, 300,000 at k = 8 758 / 772.
 constexpr int kWarpBlocks(int kc, bool trees) { return (kc == 128 || trees) ? 4 : 5; }
 
 // One query by one warp (every lane calls it with the same query). The
@@ -1378,8 +1387,8 @@ constexpr int kWarpBlocks(int kc, bool trees) { return (kc == 128 || trees) ? 4 
 // itself (the tail moved and four flag words shifted every time) and every
 // site of the descent searched for its place, a query took 40k warp
 // instructions at k = 100; 100,000 surface queries on the 1M torus took 4.01
-// ms, 2.56 now; 10,007 queries at k = 8 79 us with the sort, 68 now; 64
-// queries 19 us, 17 now (there the chain of dependent loads binds: the next
+// ms, 2.53 now; 10,007 queries at k = 8 79 us with the sort, 52 now (with
+// the one-block sort); 64 queries 19 us, 15 now (there the chain of dependent loads binds: the next
 // list's bounds are asked for before the site is put into the list). Reading
 // the lists of two sites at once, 16 lanes each, took 2.36 ms at k = 100 and
 // was slower up to k = 16; it can expand a site that would have dropped out

@@ -66,7 +66,7 @@ inline size_t defer_bytes(int64_t nq) {
 cudaError_t launch_knn_plain(const CloudDevHost& c, const PlainLaunch& L, cudaStream_t stream);
 
 // Query locality sort: a counting sort of queries by the Morton index of
-// their cell in a 64^3 grid over the cloud's bounding box.
+// their cell in a 64^3 grid over the queries' own bounding box.
 constexpr int kSortBits = 6;
 constexpr int kSortCells = 1 << (3 * kSortBits);
 constexpr int kSortTile = 1024;                       // cells per scan block
@@ -75,8 +75,14 @@ constexpr int kSortTiles = kSortCells / kSortTile;    // 256
 // (the start of a sort workspace)
 constexpr size_t kSortHistBytes = (((size_t)kSortCells * 4 + 255) & ~(size_t)255) +
                                   (((size_t)kSortTiles * 4 + 255) & ~(size_t)255) + 256;
-// Batches smaller than this skip the locality sort by default (its five
-// launches and histogram clear cost more than the order saves).
+// Batches smaller than this skip the locality sort by default. The line was
+// drawn for launches of register groups behind five sort kernels; with one warp
+// per query behind the one-block sort the order pays later still, and where
+// depends on the cloud. Whole calls, us unsorted / sorted at 4,096, 8,192,
+// 16,384 and 32,768 shuffled queries:
+//   100k-site torus    k = 8: 24/34 39/51 57/77 103/124   k = 100: 145/153 259/272 483/483 877/862
+//   1M-site torus      k = 8: 26/36 42/55 65/85 129/155   k = 100: 163/170 301/312 571/560 1025/954
+//   200k-site patches  k = 8: 111/117 172/177 177/173 305/227   k = 100: 323/293 555/433 728/613 1311/1068
 constexpr int64_t kSortMinQueries = 4096;
 // Scratch for the histogram and per-query cells (perm not included).
 size_t sort_workspace_bytes(int64_t nq);

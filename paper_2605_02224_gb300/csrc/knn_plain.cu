@@ -110,7 +110,8 @@ cudaError_t run_thread(const CloudDevHost& c, const PlainLaunch& L, cudaStream_t
 // One query per thread, candidate lists in shared memory (kcap =
 // list_slots(k) entries per thread, a warp's lists interleaved: thread l of
 // warp w owns column l of the warp's [kcap][32] keys). 256-thread blocks are
-// held to 48 registers (five blocks per SM, no spills): left alone the
+// held to 48 registers (five blocks per SM; ptxas -v spills nothing at LK = 16,
+// 16 bytes at LK = 8, 16 and 32 in their DEFER forms): left alone the
 // compiler picks either 40 registers with spills or 64, both measured
 // 5%-20% slower, and 4 or 6 blocks per SM were slower too (the torus batch at
 // k = 16: 6.45 ms with 4; 1M bumpy queries at k = 4: 0.62 ms with 4, 0.59 ms
