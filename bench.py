@@ -106,6 +106,12 @@ def _one_lane_min_queries(k: int) -> int:
     return 40960 + 1100 * k + 32768 * max(0, k - 32)
 
 
+def _default_lanes(k: int, nq: int | None = None) -> int:
+    """The lanes per query of a default launch of nq queries (None: a large one)."""
+    small = nq is not None and nq < _one_lane_min_queries(k)
+    return 32 if k >= WARP_MIN_K or small else 1
+
+
 def _query_kernel_name(lanes: int, k: int, placement: int, trees: bool = False,
                        nq: int | None = None) -> str:
     """The query kernel a plain launch of nq queries (None: a large one) with
@@ -113,16 +119,15 @@ def _query_kernel_name(lanes: int, k: int, placement: int, trees: bool = False,
     memory, one warp per query with the warp's list in shared memory from k = 48
     and in small launches; the one-warp kernel's second form walks the box trees
     of a cloud that has them)."""
-    if lanes == 0 and (k >= WARP_MIN_K or (nq is not None and nq < _one_lane_min_queries(k))):
-        lanes = 32
+    lanes = lanes or _default_lanes(k, nq)
     if lanes == 32 and placement in (0, 2):
         kc = 32 if k <= 32 else (64 if k <= 64 else 128)
         return f"knn_plain_warp_kernel<{kc}, {'true' if trees else 'false'}>"
-    if lanes in (0, 1) and placement in (0, 2):
+    if lanes == 1 and placement in (0, 2):
         threads, words = (256, 1) if k <= 32 else ((128, 2) if k <= 64 else (64, 4))
         kind = 8 if k <= 8 else (16 if k <= 16 else 0)
         return f"knn_plain_smem_kernel<{threads}, {words}, {kind}, {'true' if trees else 'false'}>"
-    if lanes in (0, 1):
+    if lanes == 1:
         return "knn_plain_thread_kernel"
     return f"knn_plain_kernel<{lanes}, S>"
 
@@ -1319,7 +1324,8 @@ def main():
                 "workload": f"torus R=1 r=0.3 sigma=1e-4, n={wl.n}, {nq} queries uniform in the "
                             f"bbox padded by 0.2, k={k}, m=n",
                 "n": wl.n, "nq": nq, "k": k, "E": st["entries"],
-                "lanes": lanes or 1,  # 0 asks for the library's default: one lane per query
+                # 0 asks for the library's default
+                "lanes": lanes or _default_lanes(k, nq),
                 "query_order": "input order" if args.no_sort else "64^3 Morton cell counting sort",
                 "l2": "flushed before every timed step (256 MB write, outside the events)",
                 "build_seconds": build_s if build_s is not None else "cached",
