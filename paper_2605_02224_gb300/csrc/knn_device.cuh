@@ -220,11 +220,11 @@ __device__ __forceinline__ void knn_query(const CloudDev& C, const Grp<G>& g, fl
   }
   for (;;) {
     const int2 rr = __ldg(C.rows + curr);
-    const int beg = rr.x, end = rr.y;
+    const uint32_t beg = rr.x, end = rr.y;  // unsigned: no overflow of base + G
     if (COUNT) qc.rows++;
     bool moved = false;
-    for (int base = beg; base < end; base += G) {
-      const int e = base + (int)g.lane;
+    for (uint32_t base = beg; base < end; base += G) {
+      const uint32_t e = base + g.lane;
       const bool valid = e < end;
       float4 ps = make_float4(0.f, 0.f, 0.f, 0.f);
       if (valid) ps = __ldg(C.ent + e);  // site and rank of the entry
@@ -268,7 +268,7 @@ __device__ __forceinline__ void knn_query(const CloudDev& C, const Grp<G>& g, fl
           qc.entries += t + 1;
           qc.coords += t;
         } else {
-          const int nv = min(G, end - base);
+          const int nv = min(G, (int)(end - base));
           qc.entries += nv;
           qc.coords += nv;
         }
@@ -301,10 +301,10 @@ __device__ __forceinline__ void knn_query(const CloudDev& C, const Grp<G>& g, fl
         if (s == psl) T.r[s] |= kDoneBit;
     }
     const int2 rr = __ldg(C.rows + site);
-    const int beg = rr.x, end = rr.y;
+    const uint32_t beg = rr.x, end = rr.y;
     if (COUNT) qc.rows++;
-    for (int base = beg; base < end; base += G) {
-      const int e = base + (int)g.lane;
+    for (uint32_t base = beg; base < end; base += G) {
+      const uint32_t e = base + g.lane;
       const bool valid = e < end;
       float4 ps = make_float4(0.f, 0.f, 0.f, 0.f);
       if (valid) ps = __ldg(C.ent + e);
@@ -328,7 +328,7 @@ __device__ __forceinline__ void knn_query(const CloudDev& C, const Grp<G>& g, fl
           qc.entries += t + 1;
           qc.coords += t;
         } else {
-          const int nv = min(G, end - base);
+          const int nv = min(G, (int)(end - base));
           qc.entries += nv;
           qc.coords += nv;
         }
@@ -1422,23 +1422,23 @@ __device__ __forceinline__ void knn_query_warp(const CloudDev& C, float qx, floa
     float dcur = sqd32(qx, qy, qz, __ldg(C.pts));
     int cur = 0;
     T.add(warp_key(dcur, 0), N, k, lane);
-    int base = rr.x;
+    uint32_t base = rr.x;  // unsigned: base + 63 does not overflow
     for (;;) {
       int to = -1;  // the site moved to
       float dto = 0.f;
-      bool over = base >= rr.y;
-      if (TREES && hub >= 0 && base - rr.x >= kHubScanFirst) {
+      bool over = base >= (uint32_t)rr.y;
+      if (TREES && hub >= 0 && (int)base - rr.x >= kHubScanFirst) {
         to = hub_first_closer(C, hub, qx, qy, qz, dcur, cur, m, lane, (uint32_t*)(list + KC), dto);
         over = true;
       } else if (!over) {
-        const int e = base + lane;
-        const float4 ps = e < rr.y ? __ldg(C.ent + e) : kNone;
+        const uint32_t e = base + lane;
+        const float4 ps = e < (uint32_t)rr.y ? __ldg(C.ent + e) : kNone;
         const int s = __float_as_int(ps.w);
         const float d = sqd32(qx, qy, qz, ps);
         // rows ascend: past the first s >= m nothing is below m
         const bool cl = s < m && strictly_closer_at(C, qx, qy, qz, d, s, dcur, cur);
         const uint32_t b = __ballot_sync(0xffffffffu, cl);
-        over = base + 32 >= rr.y || __any_sync(0xffffffffu, s >= m);
+        over = base + 32 >= (uint32_t)rr.y || __any_sync(0xffffffffu, s >= m);
         if (b) {
           const int w = __ffs((int)b) - 1;
           to = __shfl_sync(0xffffffffu, s, w);
@@ -1472,8 +1472,9 @@ __device__ __forceinline__ void knn_query_warp(const CloudDev& C, float qx, floa
       }
     }
     const int2 rr = __ldg(C.rows + site);
-    for (int e = rr.x + lane, base = rr.x; base < rr.y; base += 32, e += 32) {
-      const float4 ps = e < rr.y ? __ldg(C.ent + e) : kNone;
+    const uint32_t end = rr.y;
+    for (uint32_t e = rr.x + lane, base = rr.x; base < end; base += 32, e += 32) {
+      const float4 ps = e < end ? __ldg(C.ent + e) : kNone;
       const int s = __float_as_int(ps.w);
       const float d = sqd32(qx, qy, qz, ps);
       const uint64_t key = warp_key(d, s);
